@@ -455,9 +455,11 @@ int viscache_set_kernel_path(int path);
  * the device for that kernel's results before it reads them -- which hides
  * the gaps between them; with 0 every kernel is an ordinary launch and starts
  * only when the previous one has completed.  Results are the same either
- * way; 0 is for debugging and for timing the difference.  Calls are never
- * overlapped with work queued before them: a call's first kernel is always
- * an ordinary launch.  Errors: VC_ERR_INVALID_ARG unless on is 0 or 1.
+ * way; 0 is for debugging and for timing the difference.  A call's first
+ * kernel is an ordinary launch, so calls do not overlap with work queued
+ * before them; the one kernel of a bf16 or 4-bit decode call is a dependent
+ * launch that waits for all work before it on the stream before it reads or
+ * writes any memory.  Errors: VC_ERR_INVALID_ARG unless on is 0 or 1.
  */
 int viscache_set_dependent_launch(int on);
 

@@ -463,7 +463,7 @@ int decode_table(const vc_params* p, const std::vector<RequestPlan>& plans, int 
     const int32_t T = n_text ? n_text[r] : 0;
     if (T < 0 || T > (1 << 24)) return VC_ERR_INVALID_ARG;
   }
-  const int split = decode_split_keys(p->dtype);
+  const int split = decode_split_keys();
   tb->split = split;
   int64_t rows = 0, text = 0, units = 0, kgroups = 0;
   const int gr = kv4_group_rows();
@@ -733,7 +733,7 @@ size_t viscache_decode_workspace_size(const vc_batch* batch, const vc_params* p,
   static thread_local DecodeTable tb;
   if (decode_table(p, plans, 0, n_text, &tb) != VC_OK) return 0;   // checks the batch once
   // the largest layer's (KV head, split) units, counted as decode_table does
-  const int64_t split = decode_split_keys(p->dtype);
+  const int64_t split = decode_split_keys();
   int64_t units = 0;
   for (int l = 0; l < p->L; ++l) {
     int64_t u = 0;
@@ -769,7 +769,6 @@ int viscache_decode_attention(const vc_batch* batch, const vc_params* p, int32_t
   return cuda_status(launch_decode(tb, p->dtype, p->d, q, K_out, V_out, K_text, V_text, out,
                                    reinterpret_cast<float*>(w + dw.o_o),
                                    reinterpret_cast<float2*>(w + dw.o_ml),
-                                   reinterpret_cast<int32_t*>(w + dw.o_arr),
                                    static_cast<cudaStream_t>(stream)));
 }
 
@@ -794,12 +793,8 @@ int viscache_decode_attention_kv4(const vc_batch* batch, const vc_params* p, int
   const DecodeWs dw = decode_ws(tb.units, p->d, tb.n_req * tb.Hkv);
   const int wc = check_ws(ws, ws_bytes, dw.total);
   if (wc != VC_OK) return wc;
-  uint8_t* w = static_cast<uint8_t*>(ws);
   return cuda_status(launch_decode_kv4(tb, p->d, q, K_codes, V_codes, K_params, V_params, K_text,
-                                       V_text, out, reinterpret_cast<float*>(w + dw.o_o),
-                                       reinterpret_cast<float2*>(w + dw.o_ml),
-                                       reinterpret_cast<int32_t*>(w + dw.o_arr),
-                                       static_cast<cudaStream_t>(stream)));
+                                       V_text, out, static_cast<cudaStream_t>(stream)));
 }
 
 int viscache_kv4_sizes(const vc_batch* batch, const vc_params* p, int64_t* rows, int64_t* key_groups) {

@@ -4,35 +4,29 @@
 // over KV head g's B kept visual rows of the layer followed by its T text rows.
 //
 // A decode step reads the whole layer cache once for a handful of query rows:
-// bound by those reads.  One 256-thread CTA per unit (request, KV head, split
-// of the keys); a split's rows are staged in shared memory by 16-byte
-// asynchronous copies (the whole split in flight at once), the row's 16-byte
-// pieces XOR-permuted so that the reads hit distinct banks.
-//   decode_mma_kernel      (bf16 caches, splits of 256 keys) K rows, then V
-//                          rows, in one buffer; QK^T and PV as mma.sync
-//                          m16n8k16 tiles: keys, then output dimensions, as
-//                          M and the G <= 8 query heads as N = 8; the
-//                          split's softmax in between.  The CTA that
-//                          finishes the last split of a (request, KV head)
-//                          merges the pair's split states into the output.
-//                          Its Q4 form reads the visual rows from the 4-bit
-//                          cache: key codes and parameters loaded into
-//                          registers and expanded to bf16 rows in the same
-//                          buffer; value codes and parameters copied into
-//                          shared memory during QK and expanded after the
-//                          softmax.
-//   decode_partial_kernel  (fp32 caches, splits of 256 keys) the same steps on
-//                          CUDA cores, K then V rows in one buffer: two
-//                          threads per key pair form the logits with packed
-//                          fp32 FMAs against duplicated query values; threads
-//                          own 16-byte pieces of the V rows for a key slice;
-//                          decode_combine_kernel (one warp per request and
-//                          query head) then merges the splits.
-// Split states are the unnormalised partial output and (max, sum) per query.
+// bound by those reads.
+//   decode_tiles_kernel    (bf16 caches, and its Q4 form over the 4-bit cache)
+//                          warps stream tiles of 32 keys on the tensor cores,
+//                          a cluster of CTAs per (request, KV head) merges
+//                          them (below)
+//   decode_partial_kernel  (fp32 caches, splits of 256 keys) on CUDA cores, one
+//                          256-thread CTA per unit (request, KV head, split):
+//                          K, then V rows staged in one shared buffer by
+//                          16-byte asynchronous copies, the row's pieces
+//                          XOR-permuted so that the reads hit distinct banks;
+//                          two threads per key pair form the logits with
+//                          packed fp32 FMAs against duplicated query values;
+//                          threads own 16-byte pieces of the V rows for a key
+//                          slice; decode_combine_kernel (one warp per request
+//                          and query head) then merges the splits: the
+//                          unnormalised partial output and (max, sum) per
+//                          query.
 // A query with no keys at all (an evicted layer, no text) gets zeros.
 #include <cuda_bf16.h>
-#include <algorithm>
 #include <stdint.h>
+
+#include <algorithm>
+#include <mutex>
 
 #include "kernels.h"
 #include "profile.h"
@@ -43,7 +37,6 @@ namespace vc {
 namespace {
 
 constexpr int kSplitF = 256;                  // keys per CTA, fp32 caches (CUDA cores)
-constexpr int kSplitM = 256;                  // keys per CTA, bf16 caches (tensor cores)
 constexpr int kDecThreads = 256;
 constexpr int kDecWarps = kDecThreads / 32;
 constexpr int kGm = kDecodeMaxGroup;
@@ -267,586 +260,560 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_partial_kernel(
 }
 
 // ---------------------------------------------------------------------------
-// bf16 caches: the two contractions of a split on the tensor cores
-// (mma.sync m16n8k16, fp32 accumulation) -- keys (QK) or output dimensions
-// (PV) as M, the G <= 8 query heads of the KV head as N = 8.  The query rows
-// and the probabilities enter as bf16 high + low parts (two MMAs each), so
-// the products keep ~16 mantissa bits; K and V are exact in bf16.  Rows are
-// staged with the 16-byte pieces of row r XOR-permuted by (r & 7), which
-// makes every ldmatrix phase (8 rows, one piece column) conflict-free.
+// bf16 caches: every warp streams tiles of 32 keys of its (request, KV head)
+// on its own (no block barrier until the merge) through a ring of slots in
+// shared memory, so the loads of the next items run under the current one's
+// arithmetic.
+//
+// Both contractions are mma.sync m16n8k16 with the G <= 8 query heads as M:
+// rows 0-7 carry the bf16 high parts of the query rows (then of the
+// probabilities), rows 8-15 the low parts, so one instruction forms both
+// products and their sum keeps ~16 mantissa bits (K and V are exact in
+// bf16).  N is 8 keys (QK) or 8 output dimensions (PV).  The logits' C
+// fragment is the probabilities' A fragment, so P never leaves registers.
+// A k-step's four columns of a thread are four adjacent dimensions, half of
+// a 16-byte piece of a K row: one 16-byte shared load serves two k-steps.
+// Slots store piece c of row r at c ^ (r & 7), which makes those loads and
+// ldmatrix (V) free of bank conflicts.
+//
+// The 4-bit form (Q4) keeps codes and parameters in the slots and expands
+// them straight into B fragments: a thread's K columns as above; for PV a
+// thread takes D / 8 adjacent dimensions of its keys, one per output tile
+// (which dimension a tile's column stands for changes no sum).  The expanded
+// values are fma(code, scale, min) rounded to bf16, the rows
+// viscache_kv4_dequantize writes, and enter the same products in the same
+// order, so the result equals the bf16 kernel's over those rows bit for bit.
+//
+// A cluster of C CTAs shares a pair: warp w of the cluster takes tiles w,
+// w + 4 C, ..., each CTA merges its warps' (max, sum, output) states, sends
+// every item of four outputs to the CTA that owns it through distributed
+// shared memory, and after one cluster barrier the owners finish them.  No
+// counters or partial outputs in global memory, one kernel a call, launched
+// dependently (it waits for the previous kernel before it reads anything).
+//
+// Measured on a GB300 (28 layers as a graph, 7B shape, n = 12,544 at 19% + 512
+// text rows; before: splits of 256 keys merged through global memory): one
+// request 368 -> 147 us a step, 16 requests 785 -> 497 us (5.4 TB/s of 6.8),
+// 4-bit cache of 16 requests 925 -> 556 us.  A large layer runs at the memory
+// rate (143 MB in 24 us) plus ~3 us that the launch, the first loads and the
+// merge take; the 4-bit form is bound by instruction issue (~1,800 warp
+// instructions a tile, most of them the expansion).
 
-constexpr int kPsLd = kSplitM + 8;             // probability row stride (bf16), 16-byte skew
+constexpr int kTileKeys = 32;                  // keys per tile (one key group of the 4-bit form)
+constexpr int kWarps = 4;                      // warps per CTA
+constexpr int kMaxCluster = 16;                // CTAs per pair
+constexpr float kRise = 8.f;                   // log2 units
 
-template <int D>
-struct MmaCfg {
-  static constexpr int RB = D * 2;
-  static constexpr int PR = RB / 16;
-  static constexpr int KSTEPS = D / 16;                   // QK k-steps
-  static constexpr int DT = D / 16;                       // PV output tiles
-  static constexpr int WPT = kDecWarps / DT;              // warps per output tile
-  static constexpr int TPW = kSplitM / 16 / kDecWarps;  // QK key tiles per warp
-  static constexpr size_t BUF = (size_t)kSplitM * RB;            // one split's K, then V, rows
-  static constexpr size_t QBUF = (size_t)kGm * (RB + 16);         // query rows, 16-byte skew
-  static constexpr size_t PS = (size_t)2 * kGm * kPsLd * 2;       // P high, P low [kGm][kPsLd]
-  static constexpr size_t QF = (size_t)2 * KSTEPS * 2 * 32 * 4;   // Q^T fragments, high and low
-  static constexpr size_t RED = (size_t)(2 * kDecWarps * kGm + 2 * kGm + 4) * 4;
-  static constexpr size_t SMEM = BUF + PS + RED;
-  static_assert(TPW * 16 * kDecWarps == kSplitM, "whole QK key tiles per warp");
-  static_assert(QBUF + QF <= PS, "query rows and fragments fit the probability region");
-  static_assert(DT * WPT == kDecWarps, "output tiles divide the warps");
-  static_assert((size_t)WPT * kGm * D * 4 <= BUF, "warp partials fit a row buffer");
-  static_assert((size_t)kGm * 32 * 4 <= BUF, "merge weights fit a row buffer");
+template <int D, bool Q4>
+struct TileCfg {
+  static constexpr int RB = D * 2;                        // bytes of a bf16 row
+  static constexpr int PR = RB / 16;                      // 16-byte pieces of a row
+  static constexpr int KS = D / 16;                       // QK k-steps
+  static constexpr int NT = D / 8;                        // output tiles of 8 dimensions
+  static constexpr int ROWS = Q4 ? 16 : 32;               // bf16 rows of a ring slot
+  static constexpr int PARTS = kTileKeys / ROWS;          // slots of a tile's K (or V) rows
+  static constexpr int SLOT = ROWS * RB;
+  static constexpr int SLOTS = 3 * PARTS;                 // slots of a warp's ring (24 KB at D = 128)
+  static constexpr int RING = SLOTS * SLOT;
+  static constexpr int ITEMS = kGm * D / 4;               // outputs of a pair, four adjacent ones an item
+  // after the rings: the warps' (max, sum), the CTAs', and the CTAs' outputs of this CTA's items
+  static constexpr int TAIL = (kWarps + kMaxCluster) * kGm * 8 + (ITEMS + kMaxCluster) * 16;
+  static constexpr int SMEM = kWarps * RING + TAIL;
+  static_assert(kGm * D * 4 <= RING, "a warp's output state fits its ring");
+  // 4-bit items: codes [32][D / 2], then parameters (K: [D][2] floats, V: [32][D / 32][2])
+  static constexpr int CODES = kTileKeys * D / 2;
+  static_assert(CODES + D * 8 <= SLOT && CODES + kTileKeys * (D / 32) * 8 <= SLOT, "a 4-bit item fits a slot");
 };
-
-__device__ __forceinline__ int mma_slot(int r, int c) { return c ^ (r & 7); }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&a)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr));
-}
 __device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t (&a)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr));
+               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr) : "memory");
 }
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-
-// Unit u of the table: its request, KV head, split and row ranges.
-struct UnitRows {
-  int r, g, nk, nv, pair, nsplit;
-  int64_t vis0, txt0, u_first;   // first visual / text row, first unit of the (request, KV head)
-  int64_t kg;                    // 4-bit cache: the split's first key group
-};
-__device__ __forceinline__ UnitRows unit_rows(const DecodeTable& tb, int unit) {
-  UnitRows x;
-  x.r = find_req(tb, unit);
-  const DecodeReq& rq = tb.req[x.r];
-  const int u = unit - rq.unit0;
-  x.g = u / rq.nsplit;
-  const int s = u % rq.nsplit;
-  const int k0 = s * tb.split;
-  x.nk = max(0, min(tb.split, rq.B + rq.T - k0));
-  x.nv = max(0, min(x.nk, rq.B - k0));
-  x.vis0 = rq.vis_row0 + (int64_t)x.g * rq.B + k0;
-  x.txt0 = rq.txt_row0 + (int64_t)x.g * rq.T + (k0 + x.nv - rq.B);
-  x.pair = x.r * tb.Hkv + x.g;
-  x.nsplit = rq.nsplit;
-  x.u_first = rq.unit0 + (int64_t)x.g * rq.nsplit;
-  x.kg = rq.kg0 + (int64_t)x.g * rq.nkg + k0 / 32;
-  return x;
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp16_or_zero(uint32_t dst, const void* src, bool live) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(live ? 16u : 0u)
+               : "memory");
 }
 
-// Stage rows [first, last) of a split's rows [0, nk) (visual, then text) and
-// zeros up to the next 16-row boundary, so that the last MMA tile reads
-// finite values.  Thread t
-// copies piece column t % PR of rows t / PR + k * (threads / PR); that row
-// step is a multiple of 8, so the column's XOR slot is the same for all of the
-// thread's rows.  `zsrc` is any valid device address: the zero-filling copies
-// read no bytes.
+// Place of 16-byte piece c of bf16 row r in a slot.
 template <int D>
-__device__ __forceinline__ void stage_split(uint32_t buf_s, const __nv_bfloat16* vis,
-                                            const __nv_bfloat16* txt, int nv, int nk,
-                                            const __nv_bfloat16* zsrc, int first = 0,
-                                            int last = kSplitM) {
-  using C = MmaCfg<D>;
-  constexpr int RSTEP = kDecThreads / C::PR;
-  static_assert(RSTEP % 8 == 0, "row step keeps the XOR slot");
-  const int c = (int)threadIdx.x % C::PR, r0 = (int)threadIdx.x / C::PR;
-  const int rows = min(last, min(kSplitM, (nk + 15) & ~15));
-  const uint32_t dst0 = buf_s + r0 * C::RB + mma_slot(r0, c) * 16;
-  int r = r0;                                   // first row >= `first` in this thread's column
-  if (first > r0) r += (first - r0 + RSTEP - 1) / RSTEP * RSTEP;
-  for (; r < rows; r += RSTEP) {
-    const __nv_bfloat16* src = r < nv ? vis + (int64_t)r * D + c * 8
-                             : r < nk ? txt + (int64_t)(r - nv) * D + c * 8 : zsrc;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst0 + (r - r0) * C::RB),
-                 "l"(src), "r"(r < nk ? 16u : 0u) : "memory");
-  }
+__device__ __forceinline__ uint32_t row_at(int r, int c) {
+  return (uint32_t)(r * (D * 2) + ((c ^ (r & 7)) << 4));
 }
 
-// The G query rows of a unit (rows of the q buffer padded by 16 bytes).
-template <int D>
-__device__ __forceinline__ void stage_q(uint32_t qbuf_s, const __nv_bfloat16* qrows, int G) {
-  using C = MmaCfg<D>;
-  for (int i = (int)threadIdx.x; i < G * C::PR; i += kDecThreads) {
-    const int jj = i / C::PR, c = i % C::PR;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(qbuf_s + jj * (C::RB + 16) + c * 16),
-                 "l"(qrows + (int64_t)jj * D + c * 8) : "memory");
-  }
-}
-
-// 4-bit visual rows [0, nv) of a split expanded into bf16 rows of the
-// (XOR-permuted) row buffer: x = fma(code, scale, min) rounded to bf16, the
-// rows viscache_kv4_dequantize writes.  Thread t owns the 8-channel piece
-// c = t % PR of the PR consecutive rows (t / PR) * PR ...; those rows lie in
-// one 32-row key group, so a key thread loads its 8 channels' parameters
-// once.  Codes: D/2 bytes a row (4 bytes per piece); KEYS: parameters per
-// (key group, channel) from `par` (the split's first group); values: per
-// (row, 32-channel group) from `par` (the split's first row).
-template <int D, bool KEYS>
-__device__ __forceinline__ void expand_q4(uint8_t* buf, const uint8_t* codes, const float* par, int nv) {
-  using C = MmaCfg<D>;
-  constexpr int RPT = kSplitM * C::PR / kDecThreads;   // rows per thread (= PR)
-  static_assert(32 % RPT == 0, "a thread's rows lie in one key group");
-  const int c = (int)threadIdx.x % C::PR, r0 = (int)threadIdx.x / C::PR * RPT;
-  if (r0 >= nv) return;
-  uint32_t w[RPT];
-#pragma unroll
-  for (int i = 0; i < RPT; ++i)
-    w[i] = r0 + i < nv ? *reinterpret_cast<const uint32_t*>(codes + (size_t)(r0 + i) * (D / 2) + 4 * c) : 0u;
-  if (KEYS) {
-    float4 pk[4];                                 // (scale, min) of channels 8c + 2j, 8c + 2j + 1
-    const float4* pp = reinterpret_cast<const float4*>(par + ((size_t)(r0 >> 5) * D + 8 * c) * 2);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) pk[j] = pp[j];
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      if (r0 + i >= nv) break;
-      float x[8];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        x[2 * j] = fmaf((float)((w[i] >> (8 * j)) & 15u), pk[j].x, pk[j].y);
-        x[2 * j + 1] = fmaf((float)((w[i] >> (8 * j + 4)) & 15u), pk[j].z, pk[j].w);
-      }
-      const int r = r0 + i;
-      *reinterpret_cast<uint4*>(buf + (size_t)r * C::RB + mma_slot(r, c) * 16) =
-          make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
-    }
-  } else {
-    float2 pv[RPT];
-#pragma unroll
-    for (int i = 0; i < RPT; ++i)
-      pv[i] = r0 + i < nv ? reinterpret_cast<const float2*>(par)[(size_t)(r0 + i) * (D / 32) + (c >> 2)]
-                          : make_float2(0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      if (r0 + i >= nv) break;
-      float x[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) x[j] = fmaf((float)((w[i] >> (4 * j)) & 15u), pv[i].x, pv[i].y);
-      const int r = r0 + i;
-      *reinterpret_cast<uint4*>(buf + (size_t)r * C::RB + mma_slot(r, c) * 16) =
-          make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
-    }
-  }
-}
-
-// 4-bit value rows staged in shared memory: the split's codes at byte 0
-// (D/2 bytes a row) and their parameters after kSplitM rows of codes (one
-// (scale, min) pair per row and 32-channel group).  Rows [0, kQ4StageRows)
-// of the row buffer hold them, so the staging is used when the split's text
-// rows (which load into rows nv ...) start at or after that row.
-template <int D>
-struct Q4Stage {
-  static constexpr int CODES = kSplitM * (D / 2);
-  static constexpr int BYTES = CODES + kSplitM * (D / 32) * 8;
-  static constexpr int ROWS = (BYTES + 2 * D - 1) / (2 * D);      // bf16 rows the staging covers
-  static_assert(BYTES <= (kSplitM / 2) * 2 * D, "the staging fits the first half of the row buffer");
-};
-
-// Copy the split's value codes and parameters into the staging area (16-byte
-// asynchronous copies; all addresses are 16-byte aligned).
-template <int D>
-__device__ __forceinline__ void stage_q4_values(uint32_t buf_s, const uint8_t* codes, const float* par, int nv) {
-  using S = Q4Stage<D>;
-  const uint8_t* pp = reinterpret_cast<const uint8_t*>(par);
-  const int nc = nv * (D / 2) / 16, np = nv * (D / 32) * 8 / 16;
-  for (int i = (int)threadIdx.x; i < nc + np; i += kDecThreads) {
-    const bool is_code = i < nc;
-    const uint32_t dst = buf_s + (is_code ? 16u * i : (uint32_t)S::CODES + 16u * (i - nc));
-    const uint8_t* src = is_code ? codes + 16 * i : pp + 16 * (i - nc);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-  }
-}
-
-// Value rows [0, nv) expanded from the staging area in two steps, so that no
-// thread overwrites codes another has not read: every thread first reads its
-// rows' codes and parameters (read_q4_values), then, after a barrier, writes
-// its bf16 rows (write_q4_values).  Thread t owns the 8-channel piece
-// t % PR of rows (t / PR) * RPT ..., as in expand_q4.
-template <int D>
-struct Q4Values {
-  static constexpr int RPT = kSplitM * (D / 8) / kDecThreads;   // as expand_q4: PR = D / 8 pieces a row
-  uint32_t w[RPT];
-  float2 p[RPT];
-};
-template <int D>
-__device__ __forceinline__ void read_q4_values(const uint8_t* buf, int nv, Q4Values<D>& v) {
-  using C = MmaCfg<D>;
-  constexpr int RPT = Q4Values<D>::RPT;
-  const int c = (int)threadIdx.x % C::PR, r0 = (int)threadIdx.x / C::PR * RPT;
-  const float2* par = reinterpret_cast<const float2*>(buf + Q4Stage<D>::CODES);
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) {
-    const bool in = r0 + i < nv;
-    v.w[i] = in ? *reinterpret_cast<const uint32_t*>(buf + (size_t)(r0 + i) * (D / 2) + 4 * c) : 0u;
-    v.p[i] = in ? par[(size_t)(r0 + i) * (D / 32) + (c >> 2)] : make_float2(0.f, 0.f);
-  }
-}
-template <int D>
-__device__ __forceinline__ void write_q4_values(uint8_t* buf, int nv, const Q4Values<D>& v) {
-  using C = MmaCfg<D>;
-  constexpr int RPT = Q4Values<D>::RPT;
-  const int c = (int)threadIdx.x % C::PR, r0 = (int)threadIdx.x / C::PR * RPT;
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) {
-    if (r0 + i >= nv) break;
-    float x[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = fmaf((float)((v.w[i] >> (4 * j)) & 15u), v.p[i].x, v.p[i].y);
-    const int r = r0 + i;
-    *reinterpret_cast<uint4*>(buf + (size_t)r * C::RB + mma_slot(r, c) * 16) =
-        make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
-  }
-}
-
-// Decode kernel for bf16 caches: one CTA per unit (request, KV head, split
-// of kSplitM keys), three CTAs per SM.  The split's K rows (with the query
-// rows) load first; its V rows load into the same buffer during the softmax.
-// The CTA that completes the last split of a (request, KV head) merges that
-// pair's split states into `out`: an arrival count per pair; no CTA ever
-// waits for another.
+// Rows [0, valid) of an item (contiguous rows at src) into a slot by the
+// whole warp, zeros after them (finite values under the zero probabilities).
+// `src` is read only where rows are valid.
 template <int D, bool Q4>
-__global__ void __launch_bounds__(kDecThreads, 3) decode_mma_kernel(
-    const __grid_constant__ DecodeTable tb, const __nv_bfloat16* __restrict__ q,
+__device__ __forceinline__ void load_rows(uint32_t slot, const __nv_bfloat16* src, int valid, int lane) {
+  using C = TileCfg<D, Q4>;
+  constexpr int RPI = 32 / C::PR;               // rows per warp instruction
+  const int c = lane % C::PR, r0 = lane / C::PR;
+  const __nv_bfloat16* p = src + lane * 8;
+  if (valid >= C::ROWS) {
+#pragma unroll
+    for (int i = 0; i < C::ROWS / RPI; ++i) cp16(slot + row_at<D>(r0 + RPI * i, c), p + i * 256);
+  } else {
+#pragma unroll 2
+    for (int i = 0; i < C::ROWS / RPI; ++i) {
+      const int r = r0 + RPI * i;
+      const bool live = r < valid;
+      cp16_or_zero(slot + row_at<D>(r, c), live ? p + i * 256 : src, live);
+    }
+  }
+}
+
+// Places in a 4-bit item: byte b of code row r (D = 128: 16-byte pieces
+// flipped by bit 1 of r), and 16-byte piece p of the key parameters (flipped
+// by the thread that reads it); the value parameters lie in order.
+template <int D>
+__device__ __forceinline__ uint32_t code_at(int r, int b) {
+  return (uint32_t)(r * (D / 2) + (D == 128 ? b ^ (((r >> 1) & 1) << 5) : b));
+}
+__device__ __forceinline__ uint32_t kpar_at(int p) { return (uint32_t)((p ^ ((p >> 3) & 7)) << 4); }
+
+// `valid` rows of codes and `pars` 16-byte pieces of parameters.
+template <int D>
+__device__ __forceinline__ void load_q4(uint32_t slot, const uint8_t* codes, const void* par, int valid, int pars,
+                                        bool keys, int lane) {
+  constexpr int CP = D / 32;                    // 16-byte pieces of a code row
+  const uint8_t* cl = codes + 16 * lane;
+  const uint32_t dc = slot + code_at<D>(lane / CP, lane % CP * 16);
+  const int nc = valid * CP - lane;
+#pragma unroll
+  for (int i = 0; i < CP; ++i)                  // 32 / CP rows each: the flip is the same
+    cp16_or_zero(dc + i * 512, nc > 32 * i ? cl + 512 * i : codes, nc > 32 * i);
+  const uint8_t* pp = static_cast<const uint8_t*>(par);
+#pragma unroll
+  for (int i = 0; i < D / 64; ++i) {
+    const int p = lane + 32 * i;
+    cp16_or_zero(slot + TileCfg<D, true>::CODES + (keys ? kpar_at(p) : (uint32_t)p << 4), p < pars ? pp + 16 * p : pp,
+                 p < pars);
+  }
+}
+
+// Packed fp32 pairs kept in 64-bit registers: pairs used many times are
+// formed once.
+__device__ __forceinline__ uint64_t pair_of(float x, float y) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ uint64_t pair_of(uint32_t x, uint32_t y) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(x), "r"(y));
+  return r;
+}
+// 2^23 + byte b of x as a float's bits (asm: as intrinsics the compiler turns
+// most of these permutations into a shift and a logic operation).
+__device__ __forceinline__ uint32_t magic_byte(uint32_t x, int b) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(0x4B000000u), "r"(0x7440 | b));
+  return r;
+}
+// Byte b of x and of y as codes (exactly: 2^23 + code, minus 2^23; `bias` is
+// the pair of -2^23), then fma(code, scale, lo) rounded to bf16.
+__device__ __forceinline__ uint32_t expand_pair(uint32_t x, uint32_t y, int b, uint64_t bias, uint64_t scale,
+                                                uint64_t lo) {
+  const uint64_t c = pair_of(magic_byte(x, b), magic_byte(y, b));
+  uint64_t v;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(c), "l"(bias));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(v), "l"(scale), "l"(lo));
+  float f0, f1;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f0), "=f"(f1) : "l"(v));
+  return pack_bf16(f0, f1);
+}
+
+// Logits of the part h of a tile: s[n] += (Q high; Q low) K^T for the tile's
+// keys 8 n ... 8 n + 7.  Piece j of a thread is 2 tig + (j & 1) + 8 (j / 2).
+template <int D, bool Q4>
+__device__ __forceinline__ void qk_rows(const uint8_t* slot, const uint32_t (&qa)[D / 16][4], float (&s)[4][4],
+                                        int h, int gid, int tig) {
+  using C = TileCfg<D, Q4>;
+#pragma unroll
+  for (int j = 0; j < C::KS / 2; ++j)
+#pragma unroll
+    for (int n = 0; n < C::ROWS / 8; ++n) {
+      const uint4 u = *reinterpret_cast<const uint4*>(slot + row_at<D>(8 * n + gid, 2 * tig + (j & 1) + 8 * (j >> 1)));
+      mma_bf16(s[C::ROWS / 8 * h + n], qa[2 * j], u.x, u.y);
+      mma_bf16(s[C::ROWS / 8 * h + n], qa[2 * j + 1], u.z, u.w);
+    }
+}
+template <int D>
+__device__ __forceinline__ void qk_q4(const uint8_t* slot, const uint32_t (&qa)[D / 16][4], float (&s)[4][4],
+                                      uint64_t bias, int gid, int tig) {
+  using C = TileCfg<D, true>;
+  const uint8_t* par = slot + C::CODES + 128 * tig;
+#pragma unroll
+  for (int j = 0; j < C::KS / 2; ++j) {
+    uint64_t sc[4], lo[4];                      // the piece's channels 2 i, 2 i + 1
+    const int flip = 4 * ((j & 1) ^ (j >> 1));  // kpar_at(32 (j / 2) + 8 tig + 4 (j & 1) + i)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 f = *reinterpret_cast<const float4*>(par + 16 * (i ^ tig) + 512 * (j >> 1) + 16 * flip);
+      sc[i] = pair_of(f.x, f.z);
+      lo[i] = pair_of(f.y, f.w);
+    }
+    const uint8_t* codes = slot + code_at<D>(gid, 32 * (j >> 1) + 8 * tig);
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      const uint32_t w = *reinterpret_cast<const uint32_t*>(codes + n * 4 * D + 4 * (j & 1));
+      const uint32_t a = w & 0x0f0f0f0fu, b = (w >> 4) & 0x0f0f0f0fu;
+      uint32_t u[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) u[i] = expand_pair(a, b, i, bias, sc[i], lo[i]);
+      mma_bf16(s[n], qa[2 * j], u[0], u[1]);
+      mma_bf16(s[n], qa[2 * j + 1], u[2], u[3]);
+    }
+  }
+}
+
+// o[t] += (P high; P low) V for 16 keys, rows 16 h ... of the slot; column n
+// of output tile t is dimension 8 t + n.
+template <int D>
+__device__ __forceinline__ void pv_rows(uint32_t slot, const uint32_t (&pa)[4], int h, float (&o)[D / 8][4], int lane) {
+  const int r = 16 * h + (lane & 15), cs = lane >> 4;
+#pragma unroll
+  for (int c = 0; c < D / 8; c += 2) {
+    uint32_t v[4];
+    ldsm_x4_t(slot + row_at<D>(r, c + cs), v);
+    mma_bf16(o[c], pa, v[0], v[1]);
+    mma_bf16(o[c + 1], pa, v[2], v[3]);
+  }
+}
+// The 4-bit kernel's columns: column n of tile t is dimension (D / 8) n + t.
+template <int D>
+__device__ __forceinline__ void pv_rows_q4(const uint8_t* slot, const uint32_t (&pa)[4], float (&o)[D / 8][4], int gid,
+                                           int tig) {
+#pragma unroll
+  for (int c = 0; c < D / 64; ++c) {
+    uint32_t w[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = 2 * tig + (i & 1) + (i >> 1) * 8;
+      const uint4 u = *reinterpret_cast<const uint4*>(slot + row_at<D>(r, gid * (D / 64) + c));
+      w[i][0] = u.x; w[i][1] = u.y; w[i][2] = u.z; w[i][3] = u.w;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      mma_bf16(o[8 * c + 2 * i], pa, __byte_perm(w[0][i], w[1][i], 0x5410), __byte_perm(w[2][i], w[3][i], 0x5410));
+      mma_bf16(o[8 * c + 2 * i + 1], pa, __byte_perm(w[0][i], w[1][i], 0x7632),
+               __byte_perm(w[2][i], w[3][i], 0x7632));
+    }
+  }
+}
+template <int D>
+__device__ __forceinline__ void pv_q4(const uint8_t* slot, const uint32_t (&pa)[4], int h, float (&o)[D / 8][4],
+                                      uint64_t bias, int gid, int tig) {
+  using C = TileCfg<D, true>;
+  constexpr int WPK = D / 64;                   // code words of a thread's D / 8 dimensions
+  uint32_t w[4][WPK];                           // keys 2 tig, + 1, + 8, + 9 of the 16
+  float2 pr[4];
+  const uint8_t* codes = slot + code_at<D>(2 * tig, gid * (D / 16)) + h * 8 * D;
+  const uint8_t* par = slot + C::CODES + tig * (D / 2) + gid * D / 256 * 8 + h * 4 * D;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = (i & 1) + (i >> 1) * 8;
+    if constexpr (WPK == 2) {
+      const uint2 u = *reinterpret_cast<const uint2*>(codes + r * (D / 2));
+      w[i][0] = u.x;
+      w[i][WPK - 1] = u.y;
+    } else {
+      w[i][0] = *reinterpret_cast<const uint32_t*>(codes + r * (D / 2));
+    }
+    pr[i] = *reinterpret_cast<const float2*>(par + r * (D / 4));
+  }
+  const uint64_t s0 = pair_of(pr[0].x, pr[1].x), m0 = pair_of(pr[0].y, pr[1].y);
+  const uint64_t s1 = pair_of(pr[2].x, pr[3].x), m1 = pair_of(pr[2].y, pr[3].y);
+#pragma unroll
+  for (int k = 0; k < WPK; ++k) {
+    uint32_t a[4], b[4];                        // even and odd dimensions of the four keys
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a[i] = w[i][k] & 0x0f0f0f0fu;
+      b[i] = (w[i][k] >> 4) & 0x0f0f0f0fu;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      mma_bf16(o[8 * k + 2 * i], pa, expand_pair(a[0], a[1], i, bias, s0, m0),
+               expand_pair(a[2], a[3], i, bias, s1, m1));
+      mma_bf16(o[8 * k + 2 * i + 1], pa, expand_pair(b[0], b[1], i, bias, s0, m0),
+               expand_pair(b[2], b[3], i, bias, s1, m1));
+    }
+  }
+}
+
+// Stores to another CTA of the cluster (address from map_to_rank).
+__device__ __forceinline__ void st_cluster2(uint32_t addr, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_cluster4(uint32_t addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
+
+template <int D, bool Q4>
+__global__ void __launch_bounds__(32 * kWarps, 2) decode_tiles_kernel(
+    const __grid_constant__ DecodeTable tb, int cluster, const __nv_bfloat16* __restrict__ q,
     const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __restrict__ Vc,
     const __nv_bfloat16* __restrict__ Kt, const __nv_bfloat16* __restrict__ Vt,
     const uint8_t* __restrict__ Kq, const uint8_t* __restrict__ Vq, const float* __restrict__ Kqp,
-    const float* __restrict__ Vqp, float* __restrict__ part_o, float2* __restrict__ part_ml,
-    int32_t* __restrict__ arrivals, __nv_bfloat16* __restrict__ out) {
-  using C = MmaCfg<D>;
+    const float* __restrict__ Vqp, __nv_bfloat16* __restrict__ out) {
+  using C = TileCfg<D, Q4>;
   extern __shared__ __align__(128) uint8_t dsm[];
-  uint8_t* buf = dsm;                           // K rows, V rows, warp partials, merge weights
-  __nv_bfloat16* p_hi = reinterpret_cast<__nv_bfloat16*>(dsm + C::BUF);   // [kGm][kPsLd]
-  __nv_bfloat16* p_lo = p_hi + kGm * kPsLd;
-  // before P is written the probability region holds the query rows and fragments
-  uint8_t* qbuf = dsm + C::BUF;                                          // [kGm][RB + 16]
-  uint32_t* qf = reinterpret_cast<uint32_t*>(dsm + C::BUF + C::QBUF);     // [hi|lo][ks][hf][lane]
-  float* wmax = reinterpret_cast<float*>(dsm + C::BUF + C::PS);
-  float* wsum = wmax + kDecWarps * kGm;
-  float* cm = wsum + kDecWarps * kGm;           // merge: max, 1/sum per query
-  int* last = reinterpret_cast<int*>(cm + 2 * kGm);
-  const uint32_t buf_s = tc::smem_u32(buf), qbuf_s = tc::smem_u32(qbuf);
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int warp = (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gid = lane >> 2, tig = lane & 3;
-  const int G = tb.G;
-  const int unit = blockIdx.x;
-  const UnitRows cur = unit_rows(tb, unit);
-  const int nk = cur.nk;
-  // bf16 rows move in halves of kHalf rows, so that loads overlap the MMAs:
-  // K rows [0, kHalf) with the query rows, then K rows [kHalf, 2 kHalf); QK of
-  // the first half (tile w) runs while the second arrives; V rows [0, kHalf)
-  // load into the freed half during QK of the second half (tile w + 8), V rows
-  // [kHalf, 2 kHalf) during the softmax; PV takes the halves in turn.
-  constexpr int kHalf = kSplitM / 2;
-  static_assert(C::TPW == 2 && kHalf == 16 * kDecWarps, "QK tile h of every warp lies in half h");
-  // 4-bit: the value codes and parameters move into the first half of the row
-  // buffer while QK works on the second half (their load overlaps QK and the
-  // softmax), unless the split's text rows would land in the staging area
-  const bool q4_stage = Q4 && cur.nv >= Q4Stage<D>::ROWS;
-  if (Q4) {
-    stage_split<D>(buf_s, Kc, Kt + cur.txt0 * D, cur.nv, nk, q, cur.nv);
-    stage_q<D>(qbuf_s, q + ((int64_t)cur.r * tb.Hq + cur.g * G) * D, G);
+  const int rank = (int)blockIdx.x % cluster, pair = (int)blockIdx.x / cluster;
+  const int r = pair / tb.Hkv, g = pair % tb.Hkv, G = tb.G;
+  const int B = tb.req[r].B, T = tb.req[r].T;
+  const int64_t vis0 = tb.req[r].vis_row0 + (int64_t)g * B, txt0 = tb.req[r].txt_row0 + (int64_t)g * T;
+  const int64_t kg0 = tb.req[r].kg0 + (int64_t)g * tb.req[r].nkg;
+  const int nvt = (B + kTileKeys - 1) / kTileKeys, nt = nvt + (T + kTileKeys - 1) / kTileKeys;
+  const int first = rank * kWarps + warp, step = cluster * kWarps;
+  const int mine = nt > first ? (nt - first + step - 1) / step : 0;
+  uint8_t* ring = dsm + warp * C::RING;
+  const uint32_t ring_s = tc::smem_u32(ring);
+  float2* ml = reinterpret_cast<float2*>(dsm + kWarps * C::RING);            // [warp][query] (max, sum)
+  float2* cml = ml + kWarps * kGm;                                       // [CTA of the cluster][query]
+  float4* cout = reinterpret_cast<float4*>(cml + kMaxCluster * kGm);        // [CTA][item of this CTA]
+  if (cluster > 1) tc::cluster_arrive();        // met before the merge: every CTA has started
+
+  dep_wait();                                   // queries and cache may be the previous kernel's output
+  if (threadIdx.x == 0) dep_launch();
+
+  // Ring items, a commit group each: a tile of bf16 rows is PARTS items of K
+  // rows and as many of V rows, a 4-bit tile one of each (those come first).
+  const int q4_tiles = Q4 && nvt > first ? (nvt - first + step - 1) / step : 0;
+  auto issue = [&](int item, int slot) {
+    const uint32_t dst = ring_s + slot * C::SLOT;
+    if (Q4 && item < 2 * q4_tiles) {
+      const int t = first + (item >> 1) * step;
+      const int64_t row = vis0 + t * kTileKeys;
+      const int valid = min(kTileKeys, B - t * kTileKeys);
+      const bool v = item & 1;
+      load_q4<D>(dst, (v ? Vq : Kq) + row * (D / 2), v ? Vqp + row * (D / 32) * 2 : Kqp + (kg0 + t) * D * 2, valid,
+                 v ? valid * (D / 64) : D / 2, !v, lane);
+    } else {
+      const int e = item - 2 * q4_tiles, i = q4_tiles + e / (2 * C::PARTS);
+      if (i < mine) {
+        const int t = first + i * step;
+        const bool text = Q4 || t >= nvt, v = e & C::PARTS;
+        const int k0 = (text ? t - nvt : t) * kTileKeys + (e & (C::PARTS - 1)) * C::ROWS;
+        const __nv_bfloat16* base = text ? (v ? Vt : Kt) : (v ? Vc : Kc);
+        load_rows<D, Q4>(dst, base + ((text ? txt0 : vis0) + k0) * D, (text ? T : B) - k0, lane);
+      }
+    }
     tc::cp_async_commit();
-    expand_q4<D, true>(buf, Kq + cur.vis0 * (D / 2), Kqp + cur.kg * D * 2, cur.nv);
-    tc::cp_async_wait<0>();
-  } else {
-    stage_split<D>(buf_s, Kc + cur.vis0 * D, Kt + cur.txt0 * D, cur.nv, nk, q, 0, kHalf);
-    stage_q<D>(qbuf_s, q + ((int64_t)cur.r * tb.Hq + cur.g * G) * D, G);
-    tc::cp_async_commit();
-    stage_split<D>(buf_s, Kc + cur.vis0 * D, Kt + cur.txt0 * D, cur.nv, nk, q, kHalf);
-    tc::cp_async_commit();
-    tc::cp_async_wait<1>();                     // K rows [0, kHalf) and the query rows
-  }
-  __syncthreads();
-  // B fragments of Q^T (k = dimension, n = query) in log2 units, high + low,
-  // built once for the CTA: item (ks, hf, lane) of KSTEPS x 2 x 32
-  constexpr int ITEMS = C::KSTEPS * 2 * 32;
+  };
+#pragma unroll 1
+  for (int i = 0; i < C::SLOTS; ++i) issue(i, i);
+
+  // A fragments of the query rows in log2 units: rows 0-7 high, 8-15 low parts
+  uint32_t qa[C::KS][4];
   {
     const float c2 = tb.scale * kLog2eF;
-    for (int it = t; it < ITEMS; it += kDecThreads) {
-      const int ln = it & 31, hf = (it >> 5) & 1, ks = it >> 6;
-      const int qn = ln >> 2, qt = ln & 3;
-      float x0 = 0.f, x1 = 0.f;
-      if (qn < G) {
-        const uint32_t w = *reinterpret_cast<const uint32_t*>(
-            qbuf + qn * (C::RB + 16) + (16 * ks + 2 * qt + 8 * hf) * 2);
-        x0 = __uint_as_float(w << 16) * c2;
-        x1 = __uint_as_float(w & 0xffff0000u) * c2;
-      }
-      const float h0 = __bfloat162float(__float2bfloat16_rn(x0));
-      const float h1 = __bfloat162float(__float2bfloat16_rn(x1));
-      qf[it] = pack_bf16(h0, h1);
-      qf[ITEMS + it] = pack_bf16(x0 - h0, x1 - h1);
-    }
-  }
-  __syncthreads();
-  // QK: warp w takes key tiles w, w + 8, ... (16 keys each)
-  float sacc[C::TPW][4];
-  bool live[C::TPW];
+    const __nv_bfloat16* qr = q + ((int64_t)r * tb.Hq + g * G + min(gid, G - 1)) * D + 16 * tig;
 #pragma unroll
-  for (int h = 0; h < C::TPW; ++h) {
-    if (q4_stage && h == 1) {
-      __syncthreads();                          // K rows [0, kHalf) read: stage the value codes there
-      stage_q4_values<D>(buf_s, Vq + cur.vis0 * (D / 2), Vqp + cur.vis0 * (D / 32) * 2, cur.nv);
-      tc::cp_async_commit();
-    }
-    if (!Q4 && h == 1) {
-      __syncthreads();                          // K rows [0, kHalf) read: V rows there
-      stage_split<D>(buf_s, Vc + cur.vis0 * D, Vt + cur.txt0 * D, cur.nv, nk, q, 0, kHalf);
-      tc::cp_async_commit();
-      tc::cp_async_wait<1>();                   // K rows [kHalf, 2 kHalf)
-      __syncthreads();
-    }
-    const int mt = warp + h * kDecWarps;
-    live[h] = 16 * mt < nk;
+    for (int j = 0; j < C::KS / 2; ++j) {
+      uint4 u = *reinterpret_cast<const uint4*>(qr + 64 * (j >> 1) + 8 * (j & 1));
+      if (gid >= G) u = make_uint4(0u, 0u, 0u, 0u);
+      const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) sacc[h][i] = 0.f;
-    if (live[h]) {
-      const int row = 16 * mt + (lane & 7) + ((lane >> 3) & 1) * 8;
-#pragma unroll
-      for (int ks = 0; ks < C::KSTEPS; ++ks) {
-        uint32_t a[4];
-        ldsm_x4(buf_s + row * C::RB + mma_slot(row, 2 * ks + (lane >> 4)) * 16, a);
-        mma_bf16(sacc[h], a, qf[(2 * ks) * 32 + lane], qf[(2 * ks + 1) * 32 + lane]);
-        mma_bf16(sacc[h], a, qf[ITEMS + (2 * ks) * 32 + lane], qf[ITEMS + (2 * ks + 1) * 32 + lane]);
+      for (int i = 0; i < 4; ++i) {
+        const float x0 = __uint_as_float(w[i] << 16) * c2, x1 = __uint_as_float(w[i] & 0xffff0000u) * c2;
+        const float h0 = __bfloat162float(__float2bfloat16_rn(x0));
+        const float h1 = __bfloat162float(__float2bfloat16_rn(x1));
+        qa[2 * j + (i >> 1)][2 * (i & 1)] = pack_bf16(h0, h1);
+        qa[2 * j + (i >> 1)][2 * (i & 1) + 1] = pack_bf16(x0 - h0, x1 - h1);
       }
     }
   }
-  __syncthreads();                              // K rows, query rows, fragments read: stage V
-  if (Q4) {
-    stage_split<D>(buf_s, Vc, Vt + cur.txt0 * D, cur.nv, nk, q, cur.nv);
-    tc::cp_async_commit();
-    if (!q4_stage) expand_q4<D, false>(buf, Vq + cur.vis0 * (D / 2), Vqp + cur.vis0 * (D / 32) * 2, cur.nv);
-  } else {
-    stage_split<D>(buf_s, Vc + cur.vis0 * D, Vt + cur.txt0 * D, cur.nv, nk, q, kHalf);
-    tc::cp_async_commit();
-  }
-  // softmax over the split: lane holds keys (16 mt + gid, + 8) x queries (2 tig, + 1)
-  float x[C::TPW][4];
-  float m0 = -INFINITY, m1 = -INFINITY;
+
+  float m = -INFINITY, l = 0.f;                 // of query gid; l over this thread's keys
+  float o[C::NT][4];
 #pragma unroll
-  for (int h = 0; h < C::TPW; ++h)
+  for (int t = 0; t < C::NT; ++t)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int key = 16 * (warp + h * kDecWarps) + gid + (i >> 1) * 8;
-      x[h][i] = live[h] && key < nk ? sacc[h][i] : -INFINITY;
-      if (i & 1) m1 = fmaxf(m1, x[h][i]); else m0 = fmaxf(m0, x[h][i]);
+    for (int i = 0; i < 4; ++i) o[t][i] = 0.f;
+  const uint64_t bias = pair_of(-8388608.f, -8388608.f);
+  int slot = 0, item = 0;                       // the oldest item and its slot
+  auto refill = [&](int n) {                    // the n oldest items are read
+    __syncwarp();
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+      issue(item + C::SLOTS, slot);
+      ++item;
+      slot = slot == C::SLOTS - 1 ? 0 : slot + 1;
     }
-#pragma unroll
-  for (int o = 4; o < 32; o <<= 1) {
-    m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
-    m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-  }
-  if (gid == 0) {
-    wmax[warp * kGm + 2 * tig] = m0;
-    wmax[warp * kGm + 2 * tig + 1] = m1;
-  }
-  __syncthreads();
-  float M0 = wmax[2 * tig], M1 = wmax[2 * tig + 1];
-#pragma unroll
-  for (int w = 1; w < kDecWarps; ++w) {
-    M0 = fmaxf(M0, wmax[w * kGm + 2 * tig]);
-    M1 = fmaxf(M1, wmax[w * kGm + 2 * tig + 1]);
-  }
-  float l0 = 0.f, l1 = 0.f;
-#pragma unroll
-  for (int h = 0; h < C::TPW; ++h) {
-    if (!live[h]) continue;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int qi = 2 * tig + (i & 1);
-      const int key = 16 * (warp + h * kDecWarps) + gid + (i >> 1) * 8;
-      const float e = qi < G && key < nk ? exp2f(x[h][i] - ((i & 1) ? M1 : M0)) : 0.f;
-      if (i & 1) l1 += e; else l0 += e;
-      const __nv_bfloat16 eh = __float2bfloat16_rn(e);
-      p_hi[qi * kPsLd + key] = eh;
-      p_lo[qi * kPsLd + key] = __float2bfloat16_rn(e - __bfloat162float(eh));
-    }
-  }
-#pragma unroll
-  for (int o = 4; o < 32; o <<= 1) {
-    l0 += __shfl_xor_sync(0xffffffffu, l0, o);
-    l1 += __shfl_xor_sync(0xffffffffu, l1, o);
-  }
-  if (gid == 0) {
-    wsum[warp * kGm + 2 * tig] = l0;
-    wsum[warp * kGm + 2 * tig + 1] = l1;
-  }
-  if (Q4) tc::cp_async_wait<0>();               // V rows (and the staged codes)
-  else tc::cp_async_wait<1>();                  // V rows [0, kHalf)
-  __syncthreads();
-  if (q4_stage) {
-    Q4Values<D> qv;
-    read_q4_values<D>(buf, cur.nv, qv);
-    __syncthreads();                            // every thread has its codes: overwrite them
-    write_q4_values<D>(buf, cur.nv, qv);
-    __syncthreads();
-  }
-  if (t < G) {
-    float M = wmax[t], L = 0.f;
-#pragma unroll
-    for (int w = 0; w < kDecWarps; ++w) {
-      M = fmaxf(M, wmax[w * kGm + t]);
-      L += wsum[w * kGm + t];
-    }
-    part_ml[(int64_t)unit * kGm + t] = make_float2(M, L);
-  }
-  // PV: warp w takes output dimensions 16 (w % DT) ... and key steps w / DT, + WPT, ...
-  const int dt = warp % C::DT, kw = warp / C::DT;
-  float oacc[4] = {0.f, 0.f, 0.f, 0.f};
-  const int steps = (nk + 15) >> 4;
-  const int mi = lane >> 3;
-  auto pv_step = [&](int j) {
-    const int row = 16 * j + (lane & 7) + (mi >> 1) * 8;
-    uint32_t a[4];
-    ldsm_x4_t(buf_s + row * C::RB + mma_slot(row, 2 * dt + (mi & 1)) * 16, a);
-    const int kb = 16 * j + 2 * tig;
-    const uint32_t bh0 = *reinterpret_cast<const uint32_t*>(p_hi + gid * kPsLd + kb);
-    const uint32_t bh1 = *reinterpret_cast<const uint32_t*>(p_hi + gid * kPsLd + kb + 8);
-    const uint32_t bl0 = *reinterpret_cast<const uint32_t*>(p_lo + gid * kPsLd + kb);
-    const uint32_t bl1 = *reinterpret_cast<const uint32_t*>(p_lo + gid * kPsLd + kb + 8);
-    mma_bf16(oacc, a, bh0, bh1);
-    mma_bf16(oacc, a, bl0, bl1);
   };
-  constexpr int kHalfSteps = kHalf / 16;
-  for (int j = kw; j < min(steps, kHalfSteps); j += C::WPT) pv_step(j);
-  if (!Q4) {
-    tc::cp_async_wait<0>();                     // V rows [kHalf, 2 kHalf)
-    __syncthreads();
-  }
-  for (int j = kHalfSteps + kw % C::WPT; j < steps; j += C::WPT) pv_step(j);
-  // oacc: O[query 2 tig (+1)][dimension 16 dt + gid (+8)]
-  float* po = part_o + (int64_t)unit * kGm * D;
-  const int q0 = 2 * tig;
-  if (C::WPT == 1) {
-    float* dst = po + 16 * dt + gid;
-    if (q0 < G) {
-      dst[q0 * D] = oacc[0];
-      dst[q0 * D + 8] = oacc[2];
-    }
-    if (q0 + 1 < G) {
-      dst[(q0 + 1) * D] = oacc[1];
-      dst[(q0 + 1) * D + 8] = oacc[3];
-    }
-  } else {
-    __syncthreads();                            // V rows read: warp partials in the row buffer
-    float* wpart = reinterpret_cast<float*>(buf);   // [WPT][kGm][D]
-    float* dst = wpart + (size_t)kw * kGm * D + 16 * dt + gid;
-    dst[q0 * D] = oacc[0];
-    dst[q0 * D + 8] = oacc[2];
-    dst[(q0 + 1) * D] = oacc[1];
-    dst[(q0 + 1) * D + 8] = oacc[3];
-    __syncthreads();
-    for (int i = t; i < G * D; i += kDecThreads) {
-      float sum = 0.f;
+  // softmax of a tile's logits (keys 8 n + 2 tig, + 1 of query gid): P as A fragments
+  auto softmax = [&](const float (&s)[4][4], int valid, uint32_t (&pa)[2][4]) {
+    float x[4][2], mt = -INFINITY;
 #pragma unroll
-      for (int w = 0; w < C::WPT; ++w) sum += wpart[(size_t)w * kGm * D + i];
-      po[i] = sum;
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) x[n][e] = s[n][e] + s[n][2 + e];
+    if (valid < kTileKeys) {
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (8 * n + 2 * tig + e >= valid) x[n][e] = -INFINITY;
+    }
+#pragma unroll
+    for (int n = 0; n < 4; ++n) mt = tc::fmax3(mt, x[n][0], x[n][1]);
+    mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 1));
+    mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 2));
+    // the reference rises only past 2^kRise times the terms it allows, so a
+    // rescale of the outputs is rare; sums and products stay far below overflow
+    const bool rise = mt > m + kRise;
+    if (__any_sync(0xffffffffu, rise)) {
+      const float corr = rise ? tc::ex2(m - mt) : 1.f;
+      if (rise) m = mt;
+      l *= corr;
+#pragma unroll
+      for (int k = 0; k < C::NT; ++k)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[k][e] *= corr;
+    }
+    const float mg = m == -INFINITY ? 0.f : m;  // no finite logit yet: every term is 0
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      const float p0 = tc::ex2(x[n][0] - mg), p1 = tc::ex2(x[n][1] - mg);
+      l += p0 + p1;
+      const float h0 = __bfloat162float(__float2bfloat16_rn(p0)), h1 = __bfloat162float(__float2bfloat16_rn(p1));
+      pa[n >> 1][2 * (n & 1)] = pack_bf16(h0, h1);
+      pa[n >> 1][2 * (n & 1) + 1] = pack_bf16(p0 - h0, p1 - h1);
+    }
+  };
+  if constexpr (Q4) {
+#pragma unroll 1
+    for (int i = 0; i < q4_tiles; ++i) {
+      float s[4][4] = {};
+      uint32_t pa[2][4];
+      tc::cp_async_wait<C::SLOTS - 1>();
+      __syncwarp();
+      qk_q4<D>(ring + slot * C::SLOT, qa, s, bias, gid, tig);
+      refill(1);
+      softmax(s, B - (first + i * step) * kTileKeys, pa);
+      tc::cp_async_wait<C::SLOTS - 1>();
+      __syncwarp();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) pv_q4<D>(ring + slot * C::SLOT, pa[h], h, o, bias, gid, tig);
+      refill(1);
     }
   }
-  // arrival of this split (release: the CTA's writes, then the count); the
-  // last one merges the pair's splits
+#pragma unroll 1
+  for (int i = q4_tiles; i < mine; ++i) {
+    const int t = first + i * step;
+    float s[4][4] = {};
+    uint32_t pa[2][4];
+    tc::cp_async_wait<C::SLOTS - 1>();
+    __syncwarp();
+    qk_rows<D, Q4>(ring + slot * C::SLOT, qa, s, 0, gid, tig);
+    if constexpr (C::PARTS == 2) {
+      tc::cp_async_wait<C::SLOTS - 2>();
+      __syncwarp();
+      qk_rows<D, Q4>(ring + (slot + 1) % C::SLOTS * C::SLOT, qa, s, 1, gid, tig);
+    }
+    refill(C::PARTS);
+    softmax(s, t >= nvt ? T - (t - nvt) * kTileKeys : B - t * kTileKeys, pa);
+    tc::cp_async_wait<C::SLOTS - 1>();
+    __syncwarp();
+    if constexpr (Q4) {
+      pv_rows_q4<D>(ring + slot * C::SLOT, pa[0], o, gid, tig);
+      tc::cp_async_wait<C::SLOTS - 2>();
+      __syncwarp();
+      pv_rows_q4<D>(ring + (slot + 1) % C::SLOTS * C::SLOT, pa[1], o, gid, tig);
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) pv_rows<D>(ring_s + slot * C::SLOT, pa[h], h, o, lane);
+    }
+    refill(C::PARTS);
+  }
+  // this warp's state: (max, sum) and the unnormalised output [query][D] over its ring
+  l += __shfl_xor_sync(0xffffffffu, l, 1);
+  l += __shfl_xor_sync(0xffffffffu, l, 2);
+  if (tig == 0) ml[warp * kGm + gid] = make_float2(m, l);
+  {
+    float* po = reinterpret_cast<float*>(ring) + gid * D;
+    if constexpr (Q4) {
+#pragma unroll
+      for (int t = 0; t < C::NT; t += 4)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          *reinterpret_cast<float4*>(po + (D / 8) * (2 * tig + e) + t) =
+              make_float4(o[t][e] + o[t][2 + e], o[t + 1][e] + o[t + 1][2 + e], o[t + 2][e] + o[t + 2][2 + e],
+                          o[t + 3][e] + o[t + 3][2 + e]);
+    } else {
+#pragma unroll
+      for (int t = 0; t < C::NT; ++t)
+        *reinterpret_cast<float2*>(po + 8 * t + 2 * tig) = make_float2(o[t][0] + o[t][2], o[t][1] + o[t][3]);
+    }
+  }
   __syncthreads();
-  if (t == 0) {
-    __threadfence();
-    const int prev = atomicAdd(&arrivals[cur.pair], 1);
-    *last = prev == cur.nsplit - 1;
-  }
-  __syncthreads();
-  if (!*last) return;
-  __threadfence();
-  const int ns = cur.nsplit;
-  const float2* ml = part_ml + cur.u_first * kGm;
-  constexpr int TPQ = D / 4;
-  const int jq = t / TPQ, dq = 4 * (t % TPQ);   // thread: query jq, dimensions dq .. dq + 3
-  float* wts = reinterpret_cast<float*>(buf);   // [kGm][32] split weights
-  const float4* po4 = reinterpret_cast<const float4*>(part_o + cur.u_first * kGm * D + jq * D + dq);
-  const size_t po4_step = (size_t)kGm * D / 4;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (ns <= 32) {
-    // one load of the split states: lane s of warp jj holds split s of query jj
-    if (warp < G) {
-      const float2 v = lane < ns ? __ldcg(&ml[lane * kGm + warp]) : make_float2(-INFINITY, 0.f);
-      float M = v.x;
+  // Merge.  The CTA's warps first, four adjacent outputs an item: with one CTA
+  // that is the result; else each item goes to the CTA that owns it (CTA c
+  // owns `own` items from c own), and the (max, sum) to every CTA.
+  const int own = (C::ITEMS + cluster - 1) / cluster;
+  auto store = [&](int item, float4 v, float M, float L) {
+    // no keys: zeros; keys without a finite logit: no softmax
+    const float f = L > 0.f ? 1.f / L : M == -INFINITY && nt > 0 ? NAN : 0.f;
+    const int jj = item / (D / 4), d0 = item % (D / 4) * 4;
+    *reinterpret_cast<uint2*>(out + ((int64_t)r * tb.Hq + g * G + jj) * D + d0) =
+        make_uint2(pack_bf16(v.x * f, v.y * f), pack_bf16(v.z * f, v.w * f));
+  };
+  auto fold = [](float4& acc, float& L, float4 v, float2 st, float M) {
+    const float w = st.x == -INFINITY ? 0.f : tc::ex2(st.x - M);
+    L = fmaf(st.y, w, L);
+    acc.x = fmaf(v.x, w, acc.x);
+    acc.y = fmaf(v.y, w, acc.y);
+    acc.z = fmaf(v.z, w, acc.z);
+    acc.w = fmaf(v.w, w, acc.w);
+  };
+  if (cluster > 1) tc::cluster_wait();
+#pragma unroll 1
+  for (int item = threadIdx.x; item < G * (D / 4); item += 32 * kWarps) {
+    const int jj = item / (D / 4), d4 = item % (D / 4);
+    float M = -INFINITY, L = 0.f;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-      const float w = lane < ns && M > -INFINITY ? exp2f(v.x - M) : 0.f;
-      float L = v.y * w;
+    for (int w = 0; w < kWarps; ++w) M = fmaxf(M, ml[w * kGm + jj].x);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-      wts[warp * 32 + lane] = w;
-      if (lane == 0) cm[2 * warp + 1] = L > 0.f ? 1.f / L : 0.f;
-    }
-    __syncthreads();
-    if (jq < G) {
-#pragma unroll 16
-      for (int i = 0; i < ns; ++i) {
-        const float w = wts[jq * 32 + i];
-        const float4 v = __ldcg(po4 + i * po4_step);
-        acc.x = fmaf(v.x, w, acc.x);
-        acc.y = fmaf(v.y, w, acc.y);
-        acc.z = fmaf(v.z, w, acc.z);
-        acc.w = fmaf(v.w, w, acc.w);
-      }
-    }
-  } else {
-    if (warp < G) {
-      float M = -INFINITY;
-      for (int s = lane; s < ns; s += 32) M = fmaxf(M, __ldcg(&ml[s * kGm + warp]).x);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-      float L = 0.f;
-      if (M > -INFINITY)
-        for (int s = lane; s < ns; s += 32) {
-          const float2 v = __ldcg(&ml[s * kGm + warp]);
-          L = fmaf(v.y, exp2f(v.x - M), L);
-        }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-      if (lane == 0) {
-        cm[2 * warp] = M;
-        cm[2 * warp + 1] = L > 0.f ? 1.f / L : 0.f;
-      }
-    }
-    // 32 weights at a time
-    for (int s0 = 0; s0 < ns; s0 += 32) {
-      __syncthreads();
-      if (warp < G) {
-        const int s = s0 + lane;
-        const float M = cm[2 * warp];
-        wts[warp * 32 + lane] = s < ns && M > -INFINITY ? exp2f(__ldcg(&ml[s * kGm + warp]).x - M) : 0.f;
-      }
-      __syncthreads();
-      if (jq < G) {
-        const int cnt = min(32, ns - s0);
-#pragma unroll 16
-        for (int i = 0; i < cnt; ++i) {
-          const float w = wts[jq * 32 + i];
-          const float4 v = __ldcg(po4 + (size_t)(s0 + i) * po4_step);
-          acc.x = fmaf(v.x, w, acc.x);
-          acc.y = fmaf(v.y, w, acc.y);
-          acc.z = fmaf(v.z, w, acc.z);
-          acc.w = fmaf(v.w, w, acc.w);
-        }
-      }
+    for (int w = 0; w < kWarps; ++w)
+      fold(acc, L, *reinterpret_cast<const float4*>(dsm + w * C::RING + item * 16), ml[w * kGm + jj], M);
+    if (cluster == 1) {
+      store(item, acc, M, L);
+    } else {
+      st_cluster4(tc::map_to_rank(tc::smem_u32(cout + rank * own + item % own), item / own), acc);
+      if (d4 < cluster) st_cluster2(tc::map_to_rank(tc::smem_u32(cml + rank * kGm + jj), d4), make_float2(M, L));
     }
   }
-  if (jq < G) {
-    const float inv = cm[2 * jq + 1];
-    __nv_bfloat16* dst = out + ((int64_t)cur.r * tb.Hq + cur.g * G + jq) * D + dq;
-    *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(acc.x * inv, acc.y * inv),
-                                                pack_bf16(acc.z * inv, acc.w * inv));
+  if (cluster == 1) return;
+  __syncwarp();
+  tc::cluster_sync();                           // the cluster's states have arrived; nothing remote after it
+  for (int i = threadIdx.x; i < own; i += 32 * kWarps) {
+    const int item = rank * own + i, jj = item / (D / 4);
+    if (jj >= G) break;
+    float M = -INFINITY, L = 0.f;
+    for (int c = 0; c < cluster; ++c) M = fmaxf(M, cml[c * kGm + jj].x);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int c = 0; c < cluster; ++c) fold(acc, L, cout[c * own + i], cml[c * kGm + jj], M);
+    store(item, acc, M, L);
   }
 }
 
@@ -939,47 +906,111 @@ cudaError_t launch_decode_t(const DecodeTable& tb, const void* q, const void* Kc
   return cudaGetLastError();
 }
 
+// Cluster sizes decode_tiles_kernel is launched with.
+constexpr int kClusterSizes[] = {1, 2, 3, 4, 5, 6, 7, 8, 12, 16};
+constexpr int kClusterKinds = (int)(sizeof(kClusterSizes) / sizeof(int));
+
+// How many clusters of each size fit on a device at once (0: not launchable).
+struct DecodeFit {
+  int n[kClusterKinds] = {};
+};
+
+// CTAs per (request, KV head): the smallest cluster that gives every warp at
+// most one tile, or else the largest with which all pairs are on the device at
+// once (measured: one request, 137 tiles a pair, 10.4 us a layer with 4
+// CTAs, 7.0 with 8, 5.7 with 16; 16 requests 24.0 to 24.3 us with 2 or 4 CTAs
+// a pair and 28.5 with 6, which no longer fit at once).  The 4-bit kernel
+// takes the same sizes, so that its tiles are split and merged as the bf16
+// kernel's are.
+int decode_cluster(const DecodeTable& tb, const DecodeFit& fit) {
+  int tiles = 0;
+  for (int r = 0; r < tb.n_req; ++r)
+    tiles = std::max(tiles, (tb.req[r].B + kTileKeys - 1) / kTileKeys + (tb.req[r].T + kTileKeys - 1) / kTileKeys);
+  int best = 1;
+  for (int k = 1; k < kClusterKinds && best * kWarps < tiles; ++k)
+    if (fit.n[k] >= tb.n_req * tb.Hkv) best = kClusterSizes[k];
+  return best;
+}
+
 template <int D, bool Q4>
-cudaError_t launch_decode_mma(const DecodeTable& tb, const void* q, const void* Kc, const void* Vc,
-                              const void* Kt, const void* Vt, const uint8_t* Kq, const uint8_t* Vq,
-                              const float* Kqp, const float* Vqp, void* out, float* part_o,
-                              float2* part_ml, int32_t* arrivals, cudaStream_t st) {
-  using B16 = __nv_bfloat16;
-  if (tb.units < 1) return cudaSuccess;
-  constexpr size_t smem = MmaCfg<D>::SMEM;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(decode_mma_kernel<D, Q4>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    // the whole unified L1 as shared memory: three CTAs per SM
-    e = cudaFuncSetAttribute(decode_mma_kernel<D, Q4>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  cudaError_t e = cudaMemsetAsync(arrivals, 0, sizeof(int32_t) * tb.n_req * tb.Hkv, st);
+cudaError_t prepare_decode_tiles() {
+  auto kernel = decode_tiles_kernel<D, Q4>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TileCfg<D, Q4>::SMEM);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  // the whole unified L1 as shared memory: two CTAs per SM
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+}
+
+// Prepares both forms of the kernel on the current device at its first call
+// and returns what fits (the same for both: one shared-memory size).
+template <int D>
+cudaError_t decode_fit(DecodeFit* fit) {
+  static_assert(TileCfg<D, false>::SMEM == TileCfg<D, true>::SMEM, "both forms occupy an SM alike");
+  static bool known[64];
+  static DecodeFit fits[64];
+  static std::mutex guard;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> hold(guard);
+  if (!known[dev]) {
+    e = prepare_decode_tiles<D, false>();
+    if (e == cudaSuccess) e = prepare_decode_tiles<D, true>();
+    if (e != cudaSuccess) return e;
+    for (int k = 0; k < kClusterKinds; ++k) {
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)kClusterSizes[k];
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)kClusterSizes[k], 1, 1);
+      cfg.blockDim = dim3(32 * kWarps, 1, 1);
+      cfg.dynamicSmemBytes = TileCfg<D, false>::SMEM;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&fits[dev].n[k], decode_tiles_kernel<D, false>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        fits[dev].n[k] = 0;
+      }
+    }
+    known[dev] = true;
+  }
+  *fit = fits[dev];
+  return cudaSuccess;
+}
+
+template <int D, bool Q4>
+cudaError_t launch_decode_tiles(const DecodeTable& tb, const void* q, const void* Kc, const void* Vc,
+                                const void* Kt, const void* Vt, const uint8_t* Kq, const uint8_t* Vq,
+                                const float* Kqp, const float* Vqp, void* out, cudaStream_t st) {
+  using B16 = __nv_bfloat16;
+  if (tb.n_req < 1) return cudaSuccess;
+  DecodeFit fit;
+  const cudaError_t e = decode_fit<D>(&fit);
+  if (e != cudaSuccess) return e;
+  const int cluster = decode_cluster(tb, fit);
   ProfileScope ps(Q4 ? "decode_attn_kv4" : "decode_attn", st);
-  decode_mma_kernel<D, Q4><<<(unsigned)tb.units, kDecThreads, smem, st>>>(
-      tb, static_cast<const B16*>(q), static_cast<const B16*>(Kc), static_cast<const B16*>(Vc),
-      static_cast<const B16*>(Kt), static_cast<const B16*>(Vt), Kq, Vq, Kqp, Vqp, part_o, part_ml,
-      arrivals, static_cast<B16*>(out));
-  return cudaGetLastError();
+  return launch_dep_clusters(decode_tiles_kernel<D, Q4>, dim3((unsigned)(tb.n_req * tb.Hkv * cluster)),
+                             dim3(32 * kWarps), (size_t)TileCfg<D, Q4>::SMEM, cluster, st, tb, cluster,
+                             static_cast<const B16*>(q), static_cast<const B16*>(Kc), static_cast<const B16*>(Vc),
+                             static_cast<const B16*>(Kt), static_cast<const B16*>(Vt), Kq, Vq, Kqp, Vqp,
+                             static_cast<B16*>(out));
 }
 
 }  // namespace
 
-int decode_split_keys(int dtype) { return dtype == VC_BF16 ? kSplitM : kSplitF; }
+int decode_split_keys() { return kSplitF; }
 
 cudaError_t launch_decode(const DecodeTable& tb, int dtype, int d, const void* q, const void* Kc,
                           const void* Vc, const void* Kt, const void* Vt, void* out, float* part_o,
-                          float2* part_ml, int32_t* arrivals, cudaStream_t st) {
+                          float2* part_ml, cudaStream_t st) {
   if (dtype == VC_BF16) {
     if (d == 128)
-      return launch_decode_mma<128, false>(tb, q, Kc, Vc, Kt, Vt, nullptr, nullptr, nullptr, nullptr, out,
-                                           part_o, part_ml, arrivals, st);
-    return launch_decode_mma<64, false>(tb, q, Kc, Vc, Kt, Vt, nullptr, nullptr, nullptr, nullptr, out,
-                                        part_o, part_ml, arrivals, st);
+      return launch_decode_tiles<128, false>(tb, q, Kc, Vc, Kt, Vt, nullptr, nullptr, nullptr, nullptr, out, st);
+    return launch_decode_tiles<64, false>(tb, q, Kc, Vc, Kt, Vt, nullptr, nullptr, nullptr, nullptr, out, st);
   }
   if (d == 128) return launch_decode_t<float, 128>(tb, q, Kc, Vc, Kt, Vt, out, part_o, part_ml, st);
   return launch_decode_t<float, 64>(tb, q, Kc, Vc, Kt, Vt, out, part_o, part_ml, st);
@@ -987,13 +1018,9 @@ cudaError_t launch_decode(const DecodeTable& tb, int dtype, int d, const void* q
 
 cudaError_t launch_decode_kv4(const DecodeTable& tb, int d, const void* q, const uint8_t* Kq,
                               const uint8_t* Vq, const float* Kqp, const float* Vqp, const void* Kt,
-                              const void* Vt, void* out, float* part_o, float2* part_ml,
-                              int32_t* arrivals, cudaStream_t st) {
-  if (d == 128)
-    return launch_decode_mma<128, true>(tb, q, nullptr, nullptr, Kt, Vt, Kq, Vq, Kqp, Vqp, out, part_o,
-                                        part_ml, arrivals, st);
-  return launch_decode_mma<64, true>(tb, q, nullptr, nullptr, Kt, Vt, Kq, Vq, Kqp, Vqp, out, part_o,
-                                     part_ml, arrivals, st);
+                              const void* Vt, void* out, cudaStream_t st) {
+  if (d == 128) return launch_decode_tiles<128, true>(tb, q, nullptr, nullptr, Kt, Vt, Kq, Vq, Kqp, Vqp, out, st);
+  return launch_decode_tiles<64, true>(tb, q, nullptr, nullptr, Kt, Vt, Kq, Vq, Kqp, Vqp, out, st);
 }
 
 }  // namespace vc

@@ -33,6 +33,26 @@ cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
 }
 
+// The same for a kernel of clusters of `cluster` CTAs along x.
+template <typename... P, typename... A>
+cudaError_t launch_dep_clusters(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster,
+                                cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = g_dependent_launch.load(std::memory_order_relaxed) ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
+}
+
 // Plan-table image passed by value (kernel parameters may hold up to 32 KB).
 struct TableImage {
   alignas(16) uint8_t bytes[24 * 1024];
@@ -113,20 +133,19 @@ struct DecodeReq {
 struct DecodeTable {
   int32_t n_req, Hq, Hkv, G;
   float scale;
-  int32_t split;           // keys per split (at most decode_split_keys(dtype))
+  int32_t split;           // keys per split of the CUDA-core path (decode_split_keys())
   int32_t units;           // sum over requests of Hkv * nsplit
   DecodeReq req[kDecodeMaxReq];
 };
-int decode_split_keys(int dtype);   // the largest split a kernel takes
+int decode_split_keys();
 // Decode over the 4-bit form of the visual rows (viscache_kv4_quantize's
 // codes and parameters; bf16 query, text rows and output).
 cudaError_t launch_decode_kv4(const DecodeTable& tb, int d, const void* q, const uint8_t* Kq,
                               const uint8_t* Vq, const float* Kqp, const float* Vqp, const void* Kt,
-                              const void* Vt, void* out, float* part_o, float2* part_ml,
-                              int32_t* arrivals, cudaStream_t st);
+                              const void* Vt, void* out, cudaStream_t st);
 cudaError_t launch_decode(const DecodeTable& tb, int dtype, int d, const void* q, const void* Kc,
                           const void* Vc, const void* Kt, const void* Vt, void* out, float* part_o,
-                          float2* part_ml, int32_t* arrivals, cudaStream_t st);
+                          float2* part_ml, cudaStream_t st);
 
 // 4-bit quantisation of the compacted cache: per (request, layer) with B > 0,
 // Hkv segments of B rows starting at row0 (KV head g at row0 + g * B); a
