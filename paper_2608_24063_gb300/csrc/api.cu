@@ -702,15 +702,13 @@ int prunekv_compress(const vc_batch* batch, const vc_params* p, const void* Qw, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const float scale = p->scale == 0.f ? 1.0f / sqrtf((float)p->d) : p->scale;
   float* scores = reinterpret_cast<float*>(w + lay.o_scores);
-  int32_t* rank = reinterpret_cast<int32_t*>(w + lay.o_rank);
   int32_t* drop = reinterpret_cast<int32_t*>(w + lay.o_drop);
   cudaError_t e = launch_score(p->dtype, Qw, K, lay, scale, w, nullptr, scores, st);
   if (e != cudaSuccess) return VC_ERR_CUDA;
   const Shape sh = lay.shape(scale);
   const Tables tb = lay.tables(w);
   const int problems = lay.n_req * (p->rank_mode == VC_RANK_PER_LAYER ? p->L * p->Hkv : p->Hkv);
-  e = launch_select(sh, tb, problems, lay.max_chunks, scores, rank,
-                    reinterpret_cast<uint64_t*>(w + lay.o_chunks), idx_out, drop, st);
+  e = launch_cut(sh, tb, problems, scores, reinterpret_cast<uint64_t*>(w + lay.o_chunks), idx_out, drop, st);
   if (e != cudaSuccess) return VC_ERR_CUDA;
   e = launch_fuse(p->dtype, K, V, lay, sh, tb, idx_out, drop, p->mu, p->tau, K_out, V_out, w, st);
   return cuda_status(e);

@@ -104,6 +104,12 @@ cudaError_t launch_select(const Shape& sh, const Tables& tb, int n_problems, int
                           const float* scores, int32_t* rank, uint64_t* chunks, int32_t* keep_idx,
                           int32_t* drop_idx, cudaStream_t st);
 
+// The same lists without the ranks (the fused pass): `cuts` holds L + 1 (shared
+// ranking) or 2 (layer-specific) composites per problem; kSortChunk of them
+// always fit a problem's chunks.
+cudaError_t launch_cut(const Shape& sh, const Tables& tb, int n_problems, const float* scores, uint64_t* cuts,
+                       int32_t* keep_idx, int32_t* drop_idx, cudaStream_t st);
+
 // K_out = K[keep] (bit-exact), total_rows = Hkv * sum over requests and layers of B_l.
 cudaError_t launch_gather_k(int dtype, const void* K, const Shape& sh, const Tables& tb,
                             const int32_t* keep_idx, void* K_out, int64_t total_rows,
