@@ -111,7 +111,7 @@ struct Layout {
       q.s_off = (int64_t)per_req_problems * cu_n;
       q.out_row0 = out_rows;
       q.drop_row0 = drop_rows;
-      q.n = p.n; q.W = p.W; q.Nq = p.Nq; q.h = p.h;
+      q.n = p.n; q.W = p.W; q.Nq = p.Nq;
       q.C = (G * p.W + 255) / 256;
       q.cw = 16 * ((G * p.W + 16 * q.C - 1) / (16 * q.C));
       q.lsep_off = prows;
@@ -161,6 +161,11 @@ struct Layout {
       cu_n += p.n;
       cu_w += p.W;
     }
+    std::vector<int32_t> by_length(n_req);
+    for (int r = 0; r < n_req; ++r) by_length[r] = r;
+    std::stable_sort(by_length.begin(), by_length.end(),
+                     [&](int32_t a, int32_t b) { return plans[a].n > plans[b].n; });
+    for (int r = 0; r < n_req; ++r) req[r].by_length = by_length[r];
     row0[(size_t)n_req * L] = out_rows;
     lse_elems = (int64_t)L * Hq * cu_w;
     score_elems = (int64_t)per_req_problems * cu_n;
@@ -206,7 +211,7 @@ struct Layout {
   // the smaller S.
   void set_splits(int s) {
     S = s;
-    for (int r = 0; r < n_req; ++r) u_tc1[r + 1] = u_tc1[r] + base_tc1[r] * S;
+    for (int r = 0; r < n_req; ++r) u_tc1[r + 1] = u_tc1[r] + base_tc1[req[r].by_length] * S;
   }
   void choose_splits(int slots) {
     int best = 1;
@@ -221,10 +226,14 @@ struct Layout {
     set_splits(best);
   }
 
-  TcPlan tc_plan() const {
+  TcPlan tc_plan(std::vector<TcReq>* reqs) const {
     TcPlan t;
     t.units1 = u_tc1[n_req];
     t.units2 = u_tc2[n_req];
+    reqs->resize(n_req);
+    for (int r = 0; r < n_req; ++r) (*reqs)[r] = TcReq{u_tc2[r + 1] - u_tc2[r], req[r].Ls, req[r].C, req[r].cw};
+    t.req = reqs->data();
+    t.n_req = n_req;
     t.S = S;
     t.q_rows = q_rows;
     t.k_rows = k_rows;
@@ -310,9 +319,14 @@ cudaError_t launch_score(int dtype, const void* Qw, const void* K, Layout& lay, 
   const Shape sh = lay.shape(scale);
   const Tables tb = lay.tables(w);
   float* lse = reinterpret_cast<float*>(w + lay.o_lse);
-  if (tc)
-    return launch_score_tc(Qw, K, sh, tb, lay.tc_plan(), reinterpret_cast<float2*>(w + lay.o_part),
-                           reinterpret_cast<float*>(w + lay.o_lsep), row_lse, scores, st);
+  if (tc) {
+    // the survivors' slab (fused pass) is free until the gather
+    std::vector<TcReq> reqs;
+    const size_t slab = lay.need_vs ? (size_t)256 * lay.vs_rows : 0;
+    return launch_score_tc(Qw, K, sh, tb, lay.tc_plan(&reqs), reinterpret_cast<float2*>(w + lay.o_part),
+                           reinterpret_cast<float*>(w + lay.o_lsep), row_lse, scores, slab ? w + lay.o_vs : nullptr,
+                           slab, st);
+  }
   return launch_score_simt(dtype, Qw, K, sh, tb, lay.units_lse, lay.units_col, lse, row_lse,
                            scores, st);
 }

@@ -70,10 +70,18 @@ cudaError_t launch_score_simt(int dtype, const void* Qw, const void* K, const Sh
                               const float* lse_nat, float* scores, cudaStream_t st);
 
 // Eq. (token_score) on tcgen05 tensor cores (bf16, d = 128): lse pass (skipped when
-// lse_nat != nullptr), merge of key splits, column sums.
+// lse_nat != nullptr), merge of key splits, column sums.  `scratch` (nullable,
+// 16-byte aligned, overwritten) lets the column sums cut units between layers.
+struct TcReq {       // one request in the column-sum pass
+  int units2;        // key-tile units (Hkv * tiles, 0 when no layer is scored)
+  int layers;        // layers scored
+  int C, cw;         // chunks of a layer's rows, rows per chunk
+};
 struct TcPlan {
-  int units1;        // CTA pairs of the lse pass (sum over requests of L*Hkv*nrb*S)
-  int units2;        // CTA pairs of the column-sum pass (sum of Hkv*tiles)
+  int units1;        // units of the lse pass (sum over requests of L*Hkv*nrb*S)
+  int units2;        // units of the column-sum pass (sum of Hkv*tiles)
+  const TcReq* req;  // [n_req]
+  int n_req;
   int S;             // key splits of the lse pass
   int64_t q_rows;    // rows of the packed Qw tensor
   int64_t k_rows;    // rows of the packed K tensor
@@ -84,7 +92,7 @@ int score_tc_max_splits();
 int score_tc_pair_slots();
 cudaError_t launch_score_tc(const void* Qw, const void* K, const Shape& sh, const Tables& tb,
                             const TcPlan& tp, float2* part, float* nlse_pad, const float* lse_nat,
-                            float* scores, cudaStream_t st);
+                            float* scores, void* scratch, size_t scratch_bytes, cudaStream_t st);
 
 // bf16, d = 128: the survivors' values compacted into Vs (gather), then
 // V_out = mu V_k + (1-mu) softmax(V_k V_d^T / tau) V_d on tcgen05.  K_out =

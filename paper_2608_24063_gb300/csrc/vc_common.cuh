@@ -22,7 +22,8 @@ struct Req {                 // one request of a batch
   int64_t drop_row0;         // first drop-list row
   int64_t lsep_off;          // float offset of its chunk-padded row normalisers [L][Hkv][C*cw]
   int64_t vs_row0;           // first row of its compacted survivors' values (tensor-core fusion)
-  int32_t n, W, Nq, h;
+  int32_t n, W, Nq;
+  int32_t by_length;         // index of the request at this place when requests are ordered longest first
   int32_t C;                 // column-sum chunks of one (layer, KV head) row set, ceil(G*W/256)
   int32_t cw;                // rows per chunk: G*W spread over C chunks, rounded up to 16
   int32_t nrb;               // 256-row blocks of that row set, ceil(G*W/256)
@@ -54,7 +55,7 @@ struct Tables {              // device pointers into the workspace
   const int32_t* unit0_col;  // [n_req + 1] key-tile units of the column-sum pass
   const int32_t* unit0_fuse; // [n_req * L + 1] kept-row-tile units x Hkv of the fusion
   const int64_t* row0_out;   // [n_req * L + 1] first output row of each (request, layer)
-  const int32_t* unit0_tc1;  // [n_req + 1] CTAs of the tensor-core lse pass
+  const int32_t* unit0_tc1;  // [n_req + 1] units of the tensor-core lse pass, requests longest first
   const int32_t* unit0_tc2;  // [n_req + 1] CTAs of the tensor-core column-sum pass
   const int32_t* unit0_fuse_tc;  // [n_req * L + 1] 256-row kept tiles x Hkv (tensor-core fusion)
   const int32_t* unit0_gather;   // [n_req * L + 1] 16-row survivor blocks x Hkv (row gather)
