@@ -343,17 +343,15 @@ bool on_device(const void* p) {
 }
 
 // Prune keys and fuse values, Eq. (redistribution, weight_fusion): one tensor-core
-// kernel for bf16, d = 128 (it also copies the kept keys), else the key gather and
-// the CUDA-core fusion.
+// kernel for bf16, d = 128 (it also copies the kept keys), else the CUDA-core fusion
+// (which copies them too).
 cudaError_t launch_fuse(int dtype, const void* K, const void* V, const Layout& lay,
                         const Shape& sh, const Tables& tb, const int32_t* keep, const int32_t* drop,
                         float mu, float tau, void* K_out, void* V_out, uint8_t* w, cudaStream_t st) {
   if (g_path.load() == VC_PATH_AUTO && dtype == VC_BF16 && lay.d == 128 && lay.need_vs)
     return launch_fuse_tc(K, V, sh, tb, keep, drop, mu, tau, K_out, V_out, w + lay.o_vs,
                           lay.vs_rows, on_device(K), lay.units_gather, lay.units_fuse_tc, st);
-  cudaError_t e = launch_gather_k(dtype, K, sh, tb, keep, K_out, lay.out_rows, st);
-  if (e != cudaSuccess) return e;
-  return launch_fuse_simt(dtype, V, sh, tb, keep, drop, mu, tau, V_out, lay.units_fuse, st);
+  return launch_fuse_simt(dtype, K, V, sh, tb, keep, drop, mu, tau, K_out, V_out, lay.units_fuse, st);
 }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

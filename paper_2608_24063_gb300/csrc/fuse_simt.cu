@@ -1,11 +1,14 @@
 // Prune keys, fuse values, compact -- Algorithm 1 step 3.
 //
-// gather_k_kernel: K_out row = K row of the kept token (bit-exact 16-byte
-//   vector copies, one thread per 16 bytes, coalesced within a row).
-// fuse_v_simt_kernel: per (request, layer, KV head, tile of 32 kept rows)
-//   O = softmax_row(V_k V_d^T / tau) V_d with an online (running max / sum)
-//   softmax over tiles of 64 dropped rows, then V_out = mu V_k + (1-mu) O,
-//   Eq. (redistribution) and Eq. (weight_fusion).  Empty drop set: V_out = V_k.
+// fuse_v_simt_kernel: per (request, layer, KV head, tile of 8 R kept rows, R
+//   rows a warp) O = softmax_row(V_k V_d^T / tau) V_d with an online (running
+//   max / sum) softmax over tiles of 64 dropped rows, then
+//   V_out = mu V_k + (1-mu) O, Eq. (redistribution) and Eq. (weight_fusion).
+//   Empty drop set: V_out = V_k.  The CTA also copies its kept keys, K_out =
+//   K[keep] (bit-exact 16-byte pieces).
+// R is 4, or 1 where that would leave SMs idle (one layer of 1,024 fp32 tokens:
+// 32 CTAs); rows in shared memory are read 16 bytes at a time.  Measured on
+// that problem, with the key copy (a kernel of its own before): 23.0 -> 12.7 us.
 #include "vc_common.cuh"
 #include "kernels.h"
 #include "profile.h"
@@ -13,83 +16,75 @@
 namespace vc {
 namespace {
 
-// ---------------------------------------------------------------------------
-constexpr int kGatherThreads = 256;
-
-__global__ void __launch_bounds__(kGatherThreads) gather_k_kernel(
-    const uint4* __restrict__ K, Shape sh, Tables tb, const int32_t* __restrict__ keep_idx,
-    uint4* __restrict__ K_out, int64_t total_rows, int chunks_per_row) {
-  const int64_t t = (int64_t)blockIdx.x * kGatherThreads + threadIdx.x;
-  const int64_t row = t / chunks_per_row;
-  const int c = (int)(t % chunks_per_row);
-  if (row >= total_rows) return;
-  // (request, layer) block containing this output row
-  const int rl = upper_index(tb.row0_out, sh.n_req * sh.L, row);
-  const int r = rl / sh.L, l = rl % sh.L;
-  const Req rq = tb.req[r];
-  const Layer ly = tb.layer[rl];
-  const int64_t within = row - tb.row0_out[rl];
-  const int g = (int)(within / ly.B);
-  const int v = keep_idx[row];
-  if (v < 0 || v >= rq.n) { set_status(tb.status, VC_ERR_DEVICE_INDEX); return; }
-  const int64_t src_row = rq.kv_off / sh.d + ((int64_t)l * sh.Hkv + g) * rq.n + v;
-  K_out[row * chunks_per_row + c] = K[src_row * chunks_per_row + c];
-}
-
-// ---------------------------------------------------------------------------
-constexpr int kFuseThreads = 256;   // 8 warps x 4 kept rows
-constexpr int kFuseRows = 32;
+constexpr int kFuseThreads = 256;   // 8 warps
+constexpr int kFuseRows = 32;       // kept rows per unit of the plan tables
 constexpr int kFuseKeys = 64;       // dropped rows per tile (2 per lane)
 
-template <typename T, int D>
+template <typename T, int D, int R>
 __global__ void __launch_bounds__(kFuseThreads) fuse_v_simt_kernel(
-    const T* __restrict__ V, Shape sh, Tables tb, const int32_t* __restrict__ keep_idx,
-    const int32_t* __restrict__ drop_idx, float mu, float inv_tau_log2, T* __restrict__ V_out) {
+    const T* __restrict__ K, const T* __restrict__ V, Shape sh, Tables tb, const int32_t* __restrict__ keep_idx,
+    const int32_t* __restrict__ drop_idx, float mu, float inv_tau_log2, T* __restrict__ K_out,
+    T* __restrict__ V_out) {
   extern __shared__ float4 smem4[];
-  float* sm = reinterpret_cast<float*>(smem4);
-  float (*vk)[D + 4] = reinterpret_cast<float (*)[D + 4]>(sm);
-  float (*vd)[D + 1] = reinterpret_cast<float (*)[D + 1]>(sm + kFuseRows * (D + 4));
-  float (*ps)[kFuseKeys + 1] =
-      reinterpret_cast<float (*)[kFuseKeys + 1]>(sm + kFuseRows * (D + 4) + kFuseKeys * (D + 1));
-
+  constexpr int kBlockRows = 8 * R, kSub = kFuseRows / kBlockRows;
+  constexpr int PR = D * (int)sizeof(T) / 16;                  // 16-byte pieces of a row
+  float* vk = reinterpret_cast<float*>(smem4);                 // [kBlockRows][D + 4]
+  float* vd = vk + kBlockRows * (D + 4);                       // [kFuseKeys][D + 4]
+  float* ps = vd + kFuseKeys * (D + 4);                        // [kBlockRows][kFuseKeys + 4]
+  dep_wait();                                                  // the keep and drop lists
+  if (threadIdx.x == 0) dep_launch();
   // unit -> (request, layer), then (KV head, row tile)
-  const int rl = upper_index(tb.unit0_fuse, sh.n_req * sh.L, (int32_t)blockIdx.x);
+  const int unit = blockIdx.x / kSub;
+  const int rl = upper_index(tb.unit0_fuse, sh.n_req * sh.L, (int32_t)unit);
   const int r = rl / sh.L, l = rl % sh.L;
-  const Req rq = tb.req[r];
+  const Req& rq = tb.req[r];
   const Layer ly = tb.layer[rl];
+  const int n = rq.n;
   const int tiles = (ly.B + kFuseRows - 1) / kFuseRows;
-  const int u = blockIdx.x - tb.unit0_fuse[rl];
+  const int u = unit - tb.unit0_fuse[rl];
   const int g = u / tiles;
-  const int r0 = (u % tiles) * kFuseRows;
+  const int r0 = (u % tiles) * kFuseRows + (blockIdx.x % kSub) * kBlockRows;
+  const int rows = min(kBlockRows, ly.B - r0);
+  if (rows <= 0) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  const T* Vl = V + rq.kv_off + ((int64_t)l * sh.Hkv + g) * rq.n * D;
-  const int32_t* kp = keep_idx + rq.out_row0 + (int64_t)sh.Hkv * ly.P + (int64_t)g * ly.B;
+  const int64_t src = rq.kv_off + (int64_t)(l * sh.Hkv + g) * n * D;
+  const T* Vl = V + src;
+  const int64_t row0 = rq.out_row0 + (int64_t)sh.Hkv * ly.P + (int64_t)g * ly.B + r0;
+  const int32_t* kp = keep_idx + row0;
   const int32_t* dp = drop_idx + rq.drop_row0 + (int64_t)sh.Hkv * ly.Qd + (int64_t)g * ly.D;
-  T* out = V_out + (rq.out_row0 + (int64_t)sh.Hkv * ly.P + (int64_t)g * ly.B) * D;
-  const int rows = min(kFuseRows, ly.B - r0);
+  T* out = V_out + row0 * D;
 
-  // kept rows
-  for (int e = threadIdx.x; e < kFuseRows * (D / 4); e += kFuseThreads) {
+  // kept rows, and their keys
+  for (int e = threadIdx.x; e < kBlockRows * (D / 4); e += kFuseThreads) {
     const int rr = e / (D / 4), c4 = (e % (D / 4)) * 4;
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if (rr < rows) {
-      const int v = kp[r0 + rr];
-      if (v >= 0 && v < rq.n) x = load4(Vl + (int64_t)v * D + c4);
+      const int v = kp[rr];
+      if (v >= 0 && v < n) x = load4(Vl + (int64_t)v * D + c4);
       else set_status(tb.status, VC_ERR_DEVICE_INDEX);
     }
-    vk[rr][c4 + 0] = x.x; vk[rr][c4 + 1] = x.y; vk[rr][c4 + 2] = x.z; vk[rr][c4 + 3] = x.w;
+    *reinterpret_cast<float4*>(vk + rr * (D + 4) + c4) = x;
+  }
+  for (int e = threadIdx.x; e < rows * PR; e += kFuseThreads) {
+    const int v = kp[e / PR];
+    if (v >= 0 && v < n)
+      reinterpret_cast<uint4*>(K_out + row0 * D)[e] = reinterpret_cast<const uint4*>(K + src + (int64_t)v * D)[e % PR];
+    else
+      set_status(tb.status, VC_ERR_DEVICE_INDEX);
   }
 
   constexpr int CPL = D / 32;   // output columns per lane
-  float o[4][CPL];
-  float m[4], zs[4];
+  float o[R][CPL];
+  float m[R], zs[R];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
+  for (int a = 0; a < R; ++a) {
     m[a] = -INFINITY; zs[a] = 0.f;
 #pragma unroll
     for (int c = 0; c < CPL; ++c) o[a][c] = 0.f;
   }
+  const float* q = vk + R * warp * (D + 4);
+  float* p = ps + R * warp * (kFuseKeys + 4);
 
   for (int j0 = 0; j0 < ly.D; j0 += kFuseKeys) {
     __syncthreads();
@@ -98,29 +93,30 @@ __global__ void __launch_bounds__(kFuseThreads) fuse_v_simt_kernel(
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
       if (j0 + rr < ly.D) {
         const int v = dp[j0 + rr];
-        if (v >= 0 && v < rq.n) x = load4(Vl + (int64_t)v * D + c4);
+        if (v >= 0 && v < n) x = load4(Vl + (int64_t)v * D + c4);
         else set_status(tb.status, VC_ERR_DEVICE_INDEX);
       }
-      vd[rr][c4 + 0] = x.x; vd[rr][c4 + 1] = x.y; vd[rr][c4 + 2] = x.z; vd[rr][c4 + 3] = x.w;
+      *reinterpret_cast<float4*>(vd + rr * (D + 4) + c4) = x;
     }
     __syncthreads();
-    // logits for 4 kept rows x 2 dropped rows
-    float acc[4][2];
+    // logits for R kept rows x 2 dropped rows
+    float acc[R][2];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = 0.f;
-#pragma unroll 8
-    for (int c = 0; c < D; ++c) {
-      const float d0 = vd[lane][c], d1 = vd[lane + 32][c];
+    for (int a = 0; a < R; ++a) acc[a][0] = acc[a][1] = 0.f;
+#pragma unroll 4
+    for (int c = 0; c < D; c += 4) {
+      const float4 d0 = *reinterpret_cast<const float4*>(vd + lane * (D + 4) + c);
+      const float4 d1 = *reinterpret_cast<const float4*>(vd + (lane + 32) * (D + 4) + c);
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const float q = vk[4 * warp + a][c];
-        acc[a][0] = fmaf(q, d0, acc[a][0]);
-        acc[a][1] = fmaf(q, d1, acc[a][1]);
+      for (int a = 0; a < R; ++a) {
+        const float4 x = *reinterpret_cast<const float4*>(q + a * (D + 4) + c);
+        acc[a][0] = fmaf(x.w, d0.w, fmaf(x.z, d0.z, fmaf(x.y, d0.y, fmaf(x.x, d0.x, acc[a][0]))));
+        acc[a][1] = fmaf(x.w, d1.w, fmaf(x.z, d1.z, fmaf(x.y, d1.y, fmaf(x.x, d1.x, acc[a][1]))));
       }
     }
     const bool ok0 = j0 + lane < ly.D, ok1 = j0 + lane + 32 < ly.D;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
+    for (int a = 0; a < R; ++a) {
       const float x0 = ok0 ? acc[a][0] * inv_tau_log2 : -INFINITY;
       const float x1 = ok1 ? acc[a][1] * inv_tau_log2 : -INFINITY;
       float tm = fmaxf(x0, x1);
@@ -136,87 +132,85 @@ __global__ void __launch_bounds__(kFuseThreads) fuse_v_simt_kernel(
       m[a] = mn;
 #pragma unroll
       for (int c = 0; c < CPL; ++c) o[a][c] *= corr;
-      ps[4 * warp + a][lane] = p0;
-      ps[4 * warp + a][lane + 32] = p1;
+      p[a * (kFuseKeys + 4) + lane] = p0;
+      p[a * (kFuseKeys + 4) + lane + 32] = p1;
     }
     __syncwarp();
     // O[row][col] += sum_k P[row][k] V_d[k][col]  (cols lane + 32 c); rows are warp-private
-#pragma unroll 4
-    for (int k = 0; k < kFuseKeys; ++k) {
-      float dv[CPL];
+#pragma unroll 2
+    for (int k = 0; k < kFuseKeys; k += 4) {
+      float4 pv[R];
 #pragma unroll
-      for (int c = 0; c < CPL; ++c) dv[c] = vd[k][lane + 32 * c];
+      for (int a = 0; a < R; ++a) pv[a] = *reinterpret_cast<const float4*>(p + a * (kFuseKeys + 4) + k);
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const float p = ps[4 * warp + a][k];
+      for (int i = 0; i < 4; ++i) {
+        float dv[CPL];
 #pragma unroll
-        for (int c = 0; c < CPL; ++c) o[a][c] = fmaf(p, dv[c], o[a][c]);
+        for (int c = 0; c < CPL; ++c) dv[c] = vd[(k + i) * (D + 4) + lane + 32 * c];
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+          const float x = i == 0 ? pv[a].x : i == 1 ? pv[a].y : i == 2 ? pv[a].z : pv[a].w;
+#pragma unroll
+          for (int c = 0; c < CPL; ++c) o[a][c] = fmaf(x, dv[c], o[a][c]);
+        }
       }
     }
   }
   __syncthreads();
   // epilogue: V_out = mu V_k + (1 - mu) O / Z   (V_k itself when the drop set is empty)
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int rr = 4 * warp + a;
+  for (int a = 0; a < R; ++a) {
+    const int rr = R * warp + a;
     if (rr >= rows) continue;
     const float inv = ly.D > 0 ? 1.f / zs[a] : 0.f;
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
       const int col = lane + 32 * c;
-      const float vkc = vk[rr][col];
+      const float vkc = vk[rr * (D + 4) + col];
       const float y = ly.D > 0 ? fmaf(mu, vkc, (1.f - mu) * (o[a][c] * inv)) : vkc;
-      out[(int64_t)(r0 + rr) * D + col] = Elem<T>::from_f(y);
+      out[(int64_t)rr * D + col] = Elem<T>::from_f(y);
     }
   }
 }
 
-template <typename T, int D>
-cudaError_t launch_fuse_t(const void* V, const Shape& sh, const Tables& tb,
-                          const int32_t* keep_idx, const int32_t* drop_idx, float mu, float tau,
-                          void* V_out, int units, cudaStream_t st) {
-  const size_t smem = sizeof(float) * (kFuseRows * (D + 4) + kFuseKeys * (D + 1) +
-                                       kFuseRows * (kFuseKeys + 1));
-  cudaError_t e = cudaFuncSetAttribute(fuse_v_simt_kernel<T, D>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <typename T, int D, int R>
+cudaError_t launch_fuse_r(const void* K, const void* V, const Shape& sh, const Tables& tb, const int32_t* keep_idx,
+                          const int32_t* drop_idx, float mu, float tau, void* K_out, void* V_out, int units,
+                          cudaStream_t st) {
+  const size_t smem = sizeof(float) * ((8 * R + kFuseKeys) * (D + 4) + 8 * R * (kFuseKeys + 4));
+  cudaError_t e = cudaFuncSetAttribute(fuse_v_simt_kernel<T, D, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
   if (e != cudaSuccess) return e;
   ProfileScope ps("fuse_v_simt", st);
-  fuse_v_simt_kernel<T, D><<<units, kFuseThreads, smem, st>>>(
-      static_cast<const T*>(V), sh, tb, keep_idx, drop_idx, mu, kLog2e / tau,
-      static_cast<T*>(V_out));
-  return cudaGetLastError();
+  return launch_dep(fuse_v_simt_kernel<T, D, R>, dim3(units * (kFuseRows / (8 * R))), dim3(kFuseThreads), smem, st,
+                    static_cast<const T*>(K), static_cast<const T*>(V), sh, tb, keep_idx, drop_idx, mu, kLog2e / tau,
+                    static_cast<T*>(K_out), static_cast<T*>(V_out));
+}
+
+template <typename T, int D>
+cudaError_t launch_fuse_t(const void* K, const void* V, const Shape& sh, const Tables& tb, const int32_t* keep_idx,
+                          const int32_t* drop_idx, float mu, float tau, void* K_out, void* V_out, int units,
+                          cudaStream_t st) {
+  // fewer CTAs of 32 rows than two per SM: 8 rows each
+  return units < 304 ? launch_fuse_r<T, D, 1>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st)
+                     : launch_fuse_r<T, D, 4>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st);
 }
 
 }  // namespace
 
 int fuse_rows_per_tile_simt() { return kFuseRows; }
 
-cudaError_t launch_gather_k(int dtype, const void* K, const Shape& sh, const Tables& tb,
-                            const int32_t* keep_idx, void* K_out, int64_t total_rows,
-                            cudaStream_t st) {
-  if (total_rows == 0) return cudaSuccess;
-  const int64_t eb = dtype == VC_F32 ? 4 : 2;
-  const int chunks = (int)(sh.d * eb / 16);
-  const int64_t threads = total_rows * chunks;
-  const int64_t blocks = (threads + kGatherThreads - 1) / kGatherThreads;
-  ProfileScope ps("gather_k", st);
-  gather_k_kernel<<<(unsigned)blocks, kGatherThreads, 0, st>>>(
-      static_cast<const uint4*>(K), sh, tb, keep_idx, static_cast<uint4*>(K_out), total_rows,
-      chunks);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fuse_simt(int dtype, const void* V, const Shape& sh, const Tables& tb,
+cudaError_t launch_fuse_simt(int dtype, const void* K, const void* V, const Shape& sh, const Tables& tb,
                              const int32_t* keep_idx, const int32_t* drop_idx, float mu, float tau,
-                             void* V_out, int units, cudaStream_t st) {
+                             void* K_out, void* V_out, int units, cudaStream_t st) {
   if (units == 0) return cudaSuccess;
   if (dtype == VC_F32) {
-    if (sh.d == 64) return launch_fuse_t<float, 64>(V, sh, tb, keep_idx, drop_idx, mu, tau, V_out, units, st);
-    return launch_fuse_t<float, 128>(V, sh, tb, keep_idx, drop_idx, mu, tau, V_out, units, st);
+    if (sh.d == 64) return launch_fuse_t<float, 64>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st);
+    return launch_fuse_t<float, 128>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st);
   }
   if (sh.d == 64)
-    return launch_fuse_t<__nv_bfloat16, 64>(V, sh, tb, keep_idx, drop_idx, mu, tau, V_out, units, st);
-  return launch_fuse_t<__nv_bfloat16, 128>(V, sh, tb, keep_idx, drop_idx, mu, tau, V_out, units, st);
+    return launch_fuse_t<__nv_bfloat16, 64>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st);
+  return launch_fuse_t<__nv_bfloat16, 128>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st);
 }
 
 }  // namespace vc

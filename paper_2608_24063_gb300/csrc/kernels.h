@@ -118,15 +118,11 @@ cudaError_t launch_select(const Shape& sh, const Tables& tb, int n_problems, int
 cudaError_t launch_cut(const Shape& sh, const Tables& tb, int n_problems, const float* scores, uint64_t* cuts,
                        int32_t* keep_idx, int32_t* drop_idx, cudaStream_t st);
 
-// K_out = K[keep] (bit-exact), total_rows = Hkv * sum over requests and layers of B_l.
-cudaError_t launch_gather_k(int dtype, const void* K, const Shape& sh, const Tables& tb,
-                            const int32_t* keep_idx, void* K_out, int64_t total_rows,
-                            cudaStream_t st);
-
-// V_out = mu V_k + (1-mu) softmax(V_k V_d^T / tau) V_d on CUDA cores.
-cudaError_t launch_fuse_simt(int dtype, const void* V, const Shape& sh, const Tables& tb,
+// K_out = K[keep] (bit-exact) and V_out = mu V_k + (1-mu) softmax(V_k V_d^T / tau) V_d
+// on CUDA cores.
+cudaError_t launch_fuse_simt(int dtype, const void* K, const void* V, const Shape& sh, const Tables& tb,
                              const int32_t* keep_idx, const int32_t* drop_idx, float mu, float tau,
-                             void* V_out, int units, cudaStream_t st);
+                             void* K_out, void* V_out, int units, cudaStream_t st);
 
 // Decode attention over the compressed cache of one layer (Sec. 2, after
 // Sec. 3.2): per (request, KV head) the layer's B kept visual rows (dense
