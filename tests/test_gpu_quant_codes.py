@@ -52,3 +52,31 @@ def test_codes_equal_the_ieee_quotient(n, dtype, d):
     nb = (n + 31) // 32
     kp = kp.reshape(L * Hkv, nb, d, 2).repeat_interleave(32, dim=1)[:, :n].reshape(rows, d, 2)
     assert torch.equal(_unpack(kc.reshape(rows, -1)), _codes(xf, kp[..., 0], kp[..., 1]))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("n", [1, 7, 33, 65])
+@pytest.mark.parametrize("shift", [0, 1, 2])
+def test_codes_of_any_alignment_give_the_same_values(shift, n, dtype, d):
+    L, Hkv = 2, 3
+    batch = vc.Batch([n], [8], [(1, 1)])
+    prm = vc.make_params(L, 6, Hkv, d, vc.VC_BF16 if dtype == torch.bfloat16 else vc.VC_F32, h=L, m=(1, 1),
+                         schedule=vc.VC_SCHED_FIXED)
+    rows = L * Hkv * n
+    g = torch.Generator().manual_seed(n)
+    x = torch.randn(rows, d, generator=g).to(dtype).to(DEV)
+    kc, vcodes, kp, vp = vc.viscache_kv4_quantize(batch, prm, x, x * 2)
+
+    def moved(t):
+        buf = torch.empty(t.numel() + 16, dtype=t.dtype, device=DEV)
+        buf[shift:shift + t.numel()] = t.reshape(-1)
+        return buf[shift:shift + t.numel()].view(t.shape)
+
+    kh, vh = vc.viscache_kv4_dequantize(batch, prm, moved(kc), moved(vcodes), kp, vp, dtype=dtype)
+    s = kp.reshape(L * Hkv, (n + 31) // 32, d, 2).repeat_interleave(32, dim=1)[:, :n].reshape(rows, d, 2).double()
+    want = (_unpack(kc.reshape(rows, -1)).double() * s[..., 0] + s[..., 1]).float().to(dtype)
+    assert torch.equal(kh.reshape(rows, d), want)
+    s = vp.reshape(rows, d // 32, 2).repeat_interleave(32, dim=1).double()
+    want = (_unpack(vcodes.reshape(rows, -1)).double() * s[..., 0] + s[..., 1]).float().to(dtype)
+    assert torch.equal(vh.reshape(rows, d), want)
