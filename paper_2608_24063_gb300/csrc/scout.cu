@@ -22,21 +22,32 @@
 // Videos are independent: the batch is the data-parallel axis (one CTA each).
 //
 // Short videos (F <= 128 frames whose rows and S fit in 224 KB: the paper's 64 CLIP frames of
-// width 512) take one fused kernel instead, scout_small_kernel: one CTA per
-// video keeps the raw rows (d-major; dot products are scaled by the two
-// inverse norms afterwards) and S in shared memory, builds S
-// from 4 x 4 tiles of its upper triangle (four lanes per tile, each summing a
-// quarter of the width with packed fmas, parts added in a fixed order), and
-// runs the greedy loop inside one warp (up to four frames per lane; the warp
-// argmax is a max reduction of the score key and a min reduction of the
-// frame index; no block barriers).  Each video takes one path by its own size,
-// so a batch returns what its videos return one by one.
+// width 512) take one fused kernel instead, scout_small_kernel: a cluster of two
+// CTAs per video, each with the raw rows d-major in its shared memory (dot
+// products are scaled by the two inverse norms afterwards).  The CTAs share the
+// 4 x 4 tiles of S's upper triangle (four lanes per tile, each summing a quarter
+// of the width, parts added in a fixed order); the second writes its part into
+// the first's S through distributed shared memory.  The first CTA also computes
+// the relevances, on warps that have no tile, and runs the greedy loop inside
+// one warp (two or four frames per lane; the warp argmax is a max reduction of
+// the score key and a min reduction of the frame index; no block barriers).
+// Each video takes one path by its own size, so a batch returns what its videos
+// return one by one.
+// Bound by latency: the load, half of S's serial sums and k picks follow one
+// another.  64 videos of 64 frames (48 picks): 32.7 us with one CTA a video (64
+// of 152 SMs busy, packed fmas at a quarter of the scalar rate, transposed 4-byte
+// stores with 4-way conflicts), 20.5 us now (8.2 us
+// of it at 32 dimensions and one pick: launch, cluster start and exit).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "profile.h"
+#include "tc_common.cuh"
 #include "viscache.h"
 
 namespace vc {
@@ -62,17 +73,23 @@ struct ScoutTable {            // kernel parameter: per-video sizes and offsets
 
 constexpr int kSmallMaxFrames = 128;
 constexpr int kSmallMaxFloats = 56000;       // shared memory of the fused kernel, in floats
-constexpr int kSmallThreads = 1024;
+constexpr int kSmallThreads = 768;
 
-// d-major row stride of the fused kernel's unit rows: F rounded up to 4 plus 4
-// (16-byte aligned; the padding spreads a warp's transposed writes over banks)
+// Row strides of the fused kernel's d-major rows.  small_ld (F rounded up to 4
+// plus 4) decides by its size which videos take the kernel; wide_ld, 8 or 24
+// words mod 32, keeps the four parts of a tile's 16-byte loads on different
+// banks and is used where it still fits.
 __host__ __device__ __forceinline__ int small_ld(int F) { return ((F + 3) & ~3) + 4; }
-__host__ __device__ __forceinline__ int64_t small_floats(int F, int D) {
-  return (int64_t)D * small_ld(F) + (int64_t)F * F + D + F;
+__host__ __device__ __forceinline__ int wide_ld(int F) { return ((F + 7) & ~15) + 8; }
+__host__ __device__ __forceinline__ int64_t small_floats(int F, int D, int ld) {
+  return (int64_t)D * ld + (int64_t)F * F + D + F;
+}
+__host__ __device__ __forceinline__ int used_ld(int F, int D) {
+  return small_floats(F, D, wide_ld(F)) <= kSmallMaxFloats ? wide_ld(F) : small_ld(F);
 }
 // A video small enough for the fused kernel (the paper's 64 frames of width 512 are).
 __host__ __device__ __forceinline__ bool small_video(int F, int D) {
-  return F <= kSmallMaxFrames && small_floats(F, D) <= kSmallMaxFloats;
+  return F <= kSmallMaxFrames && small_floats(F, D, small_ld(F)) <= kSmallMaxFloats;
 }
 
 __global__ void __launch_bounds__(256) scout_norm_kernel(const float* __restrict__ H,
@@ -267,139 +284,30 @@ __global__ void __launch_bounds__(kMmrThreads, 1) scout_mmr_kernel(const __grid_
   }
 }
 
-__global__ void __launch_bounds__(kSmallThreads) scout_small_kernel(const __grid_constant__ ScoutTable tb,
-                                                                    const float* __restrict__ H,
-                                                                    const float* __restrict__ P,
-                                                                    int32_t* __restrict__ order,
-                                                                    int32_t* __restrict__ keyframes,
-                                                                    float* __restrict__ gains) {
-  extern __shared__ __align__(16) float sm[];
-  __shared__ float inv_norm[kSmallMaxFrames + 1];
-  __shared__ int pick[kSmallMaxFrames];
-  __shared__ float pick_gain[kSmallMaxFrames];
-  const int r = blockIdx.x;
-  const int F = tb.F[r], D = tb.D;
-  if (!small_video(F, D)) return;              // the three-kernel path takes it
-  const int k = tb.k[r], ld = small_ld(F);
-  const float lam = tb.lam;
-  float* hT = sm;                              // [D][ld] unit rows, d-major
-  float* S = hT + (size_t)D * ld;              // [F][F]
-  float* tn = S + (size_t)F * F;               // [D] unit prompt
-  float* rel = tn + D;                         // [F] relevance
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const float* h = H + tb.h_off[r] * D;
-  // raw rows into shared memory (d-major; the prompt as row F) and each
-  // row's inverse norm; dot products of raw rows are scaled by both inverse
-  // norms afterwards (one pass over global memory, no scaling pass)
-  for (int row = warp; row <= F; row += kSmallThreads / 32) {
-    const float* src = row < F ? h + (int64_t)row * D : P + (int64_t)r * D;
-    float ss = 0.f;
-#pragma unroll 8
-    for (int j = lane; j < D; j += 32) {
-      const float x = src[j];
-      ss = fmaf(x, x, ss);
-      if (row < F) hT[(size_t)j * ld + row] = x;
-      else tn[j] = x;
-    }
+// The greedy loop of one warp: the lane holds frames lane, lane + 32, ... (J of
+// them); pick[i] and pick_gain[i] get the i-th frame and its score.
+template <int J>
+__device__ __forceinline__ void pick_frames(const float* S, const float* rel, int F, int k, float lam, int* pick,
+                                            float* pick_gain, bool (&sel)[kSmallMaxFrames / 32]) {
+  const int lane = threadIdx.x & 31;
+  float lr[J], red[J];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (lane == 0) inv_norm[row] = ss > 0.f ? 1.f / sqrtf(ss) : 0.f;
-  }
-  __syncthreads();
-  // S = hn hn^T: 4 x 4 tiles of the upper triangle, mirrored.  Four adjacent
-  // lanes share a tile, lane part p summing widths p, p+4, ... (four frames
-  // per 16-byte load, two products per packed fma); the parts are added as
-  // (p0 + p1) + (p2 + p3) by two shuffles.
-  const int nt = (F + 3) / 4;
-  const int ntri = nt * (nt + 1) / 2;
-  for (int item = threadIdx.x; item < 4 * ((ntri + 7) / 8) * 8; item += kSmallThreads) {
-    const int t = item >> 2, part = item & 3;
-    const bool live = t < ntri;
-    int a = 0, rem = live ? t : 0;
-    while (rem >= nt - a) {
-      rem -= nt - a;
-      ++a;
-    }
-    const int i0 = a * 4, j0 = (a + rem) * 4;
-    float2 acc[4][2];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u][0] = acc[u][1] = make_float2(0.f, 0.f);
-    if (live) {
-#pragma unroll 4
-      for (int d = part; d < D; d += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(hT + (size_t)d * ld + i0);
-        const float4 y = *reinterpret_cast<const float4*>(hT + (size_t)d * ld + j0);
-        const float xs[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          acc[u][0] = __ffma2_rn(make_float2(xs[u], xs[u]), make_float2(y.x, y.y), acc[u][0]);
-          acc[u][1] = __ffma2_rn(make_float2(xs[u], xs[u]), make_float2(y.z, y.w), acc[u][1]);
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        float2 w = acc[u][v];
-        w.x += __shfl_xor_sync(0xffffffffu, w.x, 1);
-        w.y += __shfl_xor_sync(0xffffffffu, w.y, 1);
-        w.x += __shfl_xor_sync(0xffffffffu, w.x, 2);
-        w.y += __shfl_xor_sync(0xffffffffu, w.y, 2);
-        acc[u][v] = w;
-      }
-    if (live && part == 0) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float v4[4] = {acc[u][0].x, acc[u][0].y, acc[u][1].x, acc[u][1].y};
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const int i = i0 + u, j = j0 + v;
-          if (i < F && j < F) {
-            const float c = (v4[v] * inv_norm[i]) * inv_norm[j];
-            S[(size_t)i * F + j] = c;
-            S[(size_t)j * F + i] = c;
-          }
-        }
-      }
-    }
-  }
-  // relevance: four lanes per frame, parts combined as for S
-  for (int item = threadIdx.x; item < 4 * ((F + 7) / 8) * 8; item += kSmallThreads) {
-    const int f = item >> 2, part = item & 3;
-    float acc = 0.f;
-    if (f < F)
-      for (int d = part; d < D; d += 4) acc = fmaf(hT[(size_t)d * ld + f], tn[d], acc);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-    if (f < F && part == 0) rel[f] = (acc * inv_norm[f]) * inv_norm[F];
-  }
-  __syncthreads();
-  if (warp != 0) return;
-  // greedy loop in warp 0: lane holds frames lane, lane + 32, ...
-  constexpr int kLaneFrames = kSmallMaxFrames / 32;
-  float rl[kLaneFrames], red[kLaneFrames];
-  bool sel[kLaneFrames];
-#pragma unroll
-  for (int j = 0; j < kLaneFrames; ++j) {
+  for (int j = 0; j < J; ++j) {
     const int f = lane + 32 * j;
-    rl[j] = f < F ? rel[f] : 0.f;
+    lr[j] = f < F ? lam * rel[f] : 0.f;
     red[j] = 0.f;                                // empty selected set: no redundancy
     sel[j] = f >= F;                             // frames past F are never picked
   }
-  const int o0 = tb.k_off[r];
   for (int i = 0; i < k; ++i) {
     // this lane's best frame (highest score, then lowest index), then the
     // warp's: the highest score key, and the lowest frame holding it
     uint32_t kb = 0, fb = 0xffffffffu;
 #pragma unroll
-    for (int j = 0; j < kLaneFrames; ++j) {
-      if (!sel[j]) {
-        const uint32_t key = ord_key(fmaf(-(1.f - lam), red[j], lam * rl[j]));
-        if (key > kb) {
-          kb = key;
-          fb = (uint32_t)(lane + 32 * j);
-        }
+    for (int j = 0; j < J; ++j) {
+      const uint32_t key = sel[j] ? 0u : ord_key(fmaf(-(1.f - lam), red[j], lr[j]));
+      if (key > kb) {
+        kb = key;
+        fb = (uint32_t)(lane + 32 * j);
       }
     }
     const uint32_t kmax = __reduce_max_sync(0xffffffffu, kb);
@@ -410,7 +318,7 @@ __global__ void __launch_bounds__(kSmallThreads) scout_small_kernel(const __grid
     }
     const float* row = S + (size_t)fs * F;
 #pragma unroll
-    for (int j = 0; j < kLaneFrames; ++j) {
+    for (int j = 0; j < J; ++j) {
       const int f = lane + 32 * j;
       if (f < F) {
         red[j] = i == 0 ? row[f] : fmaxf(red[j], row[f]);
@@ -418,6 +326,137 @@ __global__ void __launch_bounds__(kSmallThreads) scout_small_kernel(const __grid
       }
     }
   }
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSmallThreads, 1)
+    scout_small_kernel(const __grid_constant__ ScoutTable tb, const float* __restrict__ H, const float* __restrict__ P,
+                       int32_t* __restrict__ order, int32_t* __restrict__ keyframes, float* __restrict__ gains) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ float inv_norm[kSmallMaxFrames + 1];
+  __shared__ int pick[kSmallMaxFrames];
+  __shared__ float pick_gain[kSmallMaxFrames];
+  const int r = blockIdx.x >> 1, rank = blockIdx.x & 1;
+  const int F = tb.F[r], D = tb.D;
+  if (!small_video(F, D)) return;              // the three-kernel path takes it (both CTAs leave)
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  tc::cluster_arrive();                            // "started": waited for before S is written remotely
+  const int k = tb.k[r], ld = used_ld(F, D);
+  const float lam = tb.lam;
+  float* hT = sm;                              // [D][ld] rows, d-major
+  float* S = hT + (size_t)D * ld;              // [F][F] (the first CTA's is used)
+  float* tn = S + (size_t)F * F;               // [D] prompt
+  float* rel = tn + D;                         // [F] relevance
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float* h = H + tb.h_off[r] * D;
+  const int nt = (F + 3) / 4;
+  // raw rows into shared memory (four rows of a warp as one 16-byte piece per
+  // dimension; the prompt as group nt) and each row's inverse norm
+  for (int q = warp; q <= nt; q += kSmallThreads / 32) {
+    float ss[4] = {};
+    const float* src[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) src[u] = q < nt ? (4 * q + u < F ? h + (int64_t)(4 * q + u) * D : nullptr)
+                                               : (u == 0 ? P + (int64_t)r * D : nullptr);
+#pragma unroll 8
+    for (int j = lane; j < D; j += 32) {
+      float x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = src[u] ? src[u][j] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ss[u] = fmaf(x[u], x[u], ss[u]);
+      if (q < nt) *reinterpret_cast<float4*>(hT + (size_t)j * ld + 4 * q) = make_float4(x[0], x[1], x[2], x[3]);
+      else tn[j] = x[0];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) ss[u] += __shfl_xor_sync(0xffffffffu, ss[u], o);
+      const int row = q < nt ? 4 * q + u : F + u;
+      if (lane == 0 && row <= F && (q == nt || row < F)) inv_norm[row] = ss[u] > 0.f ? 1.f / sqrtf(ss[u]) : 0.f;
+    }
+  }
+  __syncthreads();
+  tc::cluster_wait();
+  float* S0 = cluster.map_shared_rank(S, 0);
+  // S = hn hn^T: 4 x 4 tiles of the upper triangle, mirrored; this CTA takes
+  // every second one.  Four adjacent lanes share a tile, lane part p summing
+  // widths p, p+4, ...; the parts are added as (p0 + p1) + (p2 + p3) by two
+  // shuffles, and lane p scales and writes the tile's row p.
+  const int ntri = nt * (nt + 1) / 2;
+  const int mine = (ntri + 1 - rank) / 2;
+  for (int item = threadIdx.x; item < 4 * ((mine + 7) / 8) * 8; item += kSmallThreads) {
+    const int part = item & 3;
+    const bool live = (item >> 2) < mine;
+    int a = 0, rem = live ? 2 * (item >> 2) + rank : 0;
+    while (rem >= nt - a) {
+      rem -= nt - a;
+      ++a;
+    }
+    const int i0 = a * 4, j0 = (a + rem) * 4;
+    float acc[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+    if (live) {
+#pragma unroll 8
+      for (int d = part; d < D; d += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(hT + (size_t)d * ld + i0);
+        const float4 y = *reinterpret_cast<const float4*>(hT + (size_t)d * ld + j0);
+        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(xs[u], ys[v], acc[u][v]);
+      }
+    }
+    float out[4] = {};                         // row `part` of the tile
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        float w = acc[u][v];
+        w += __shfl_xor_sync(0xffffffffu, w, 1);
+        w += __shfl_xor_sync(0xffffffffu, w, 2);
+        if (part == u) out[v] = w;
+      }
+    const int i = i0 + part;
+    if (live && i < F) {
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int j = j0 + v;
+        if (j < F && (i0 != j0 || j <= i)) {   // a diagonal tile's pairs once, the larger index first
+          const float c = (out[v] * inv_norm[i]) * inv_norm[j];
+          S0[(size_t)i * F + j] = c;
+          S0[(size_t)j * F + i] = c;
+        }
+      }
+    }
+  }
+  // relevance, from the last warp down (the tiles fill from the first): four
+  // lanes per frame, parts combined as for S
+  if (rank == 0)
+    for (int item = kSmallThreads - 32 - 32 * warp + lane; item < 4 * ((F + 7) / 8) * 8; item += kSmallThreads) {
+      const int f = item >> 2, part = item & 3;
+      float acc = 0.f;
+      if (f < F) {
+#pragma unroll 8
+        for (int d = part; d < D; d += 4) acc = fmaf(hT[(size_t)d * ld + f], tn[d], acc);
+      }
+      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+      if (f < F && part == 0) rel[f] = (acc * inv_norm[f]) * inv_norm[F];
+    }
+  __syncwarp();
+  tc::cluster_arrive();
+  tc::cluster_wait();                              // S and the relevances are complete in the first CTA
+  if (rank != 0 || warp != 0) return;
+  // greedy loop in warp 0: lane holds frames lane, lane + 32, ...
+  constexpr int kLaneFrames = kSmallMaxFrames / 32;
+  bool sel[kLaneFrames] = {};
+  if (F <= 64) pick_frames<2>(S, rel, F, k, lam, pick, pick_gain, sel);
+  else pick_frames<kLaneFrames>(S, rel, F, k, lam, pick, pick_gain, sel);
+  const int o0 = tb.k_off[r];
   __syncwarp();
   for (int i = lane; i < k; i += 32) {
     order[o0 + i] = pick[i];
@@ -517,18 +556,19 @@ extern "C" int viscache_scout_mmr(const float* H, const float* prompt, int32_t n
   float* S = reinterpret_cast<float*>(w + lay.o_s);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // each video goes to the fused kernel or to the three-kernel path by its size
-  int fmax_small = 0, fmax_large = 0;
+  int fmax_large = 0;
+  int64_t floats_small = 0;
   for (int r = 0; r < n_req; ++r) {
-    if (small_video(tb.F[r], D)) fmax_small = tb.F[r] > fmax_small ? tb.F[r] : fmax_small;
-    else fmax_large = tb.F[r] > fmax_large ? tb.F[r] : fmax_large;
+    if (small_video(tb.F[r], D)) floats_small = std::max(floats_small, small_floats(tb.F[r], D, used_ld(tb.F[r], D)));
+    else fmax_large = std::max(fmax_large, tb.F[r]);
   }
-  if (fmax_small > 0) {
+  if (floats_small > 0) {
     ProfileScope ps("scout_small", st);
-    const size_t smem = sizeof(float) * (size_t)small_floats(fmax_small, D);
+    const size_t smem = sizeof(float) * (size_t)floats_small;
     if (cudaFuncSetAttribute(scout_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
       return VC_ERR_CUDA;
-    scout_small_kernel<<<(unsigned)n_req, kSmallThreads, smem, st>>>(tb, H, prompt, order_out, keyframes_out,
+    scout_small_kernel<<<2u * (unsigned)n_req, kSmallThreads, smem, st>>>(tb, H, prompt, order_out, keyframes_out,
                                                                     gains_out);
     if (cudaGetLastError() != cudaSuccess) return VC_ERR_CUDA;
   }
