@@ -294,10 +294,11 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_partial_kernel(
 // Measured on a GB300 (28 layers as a graph, 7B shape, n = 12,544 at 19% + 512
 // text rows; before: splits of 256 keys merged through global memory): one
 // request 368 -> 147 us a step, 16 requests 785 -> 497 us (5.4 TB/s of 6.8),
-// 4-bit cache of 16 requests 925 -> 556 us.  A large layer runs at the memory
+// 4-bit cache of 16 requests 925 -> 528 us (556 with packed fp32 expansion).  A large layer runs at the memory
 // rate (143 MB in 24 us) plus ~3 us that the launch, the first loads and the
-// merge take; the 4-bit form is bound by instruction issue (~1,800 warp
-// instructions a tile, most of them the expansion).
+// merge take; the 4-bit form is bound by instruction latency and
+// issue (~1,650 warp instructions a tile, most of them the expansion, on two
+// warps a scheduler).
 
 constexpr int kTileKeys = 32;                  // keys per tile (one key group of the 4-bit form)
 constexpr int kWarps = 4;                      // warps per CTA
@@ -405,18 +406,6 @@ __device__ __forceinline__ void load_q4(uint32_t slot, const uint8_t* codes, con
   }
 }
 
-// Packed fp32 pairs kept in 64-bit registers: pairs used many times are
-// formed once.
-__device__ __forceinline__ uint64_t pair_of(float x, float y) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ uint64_t pair_of(uint32_t x, uint32_t y) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(x), "r"(y));
-  return r;
-}
 // 2^23 + byte b of x as a float's bits (asm: as intrinsics the compiler turns
 // most of these permutations into a shift and a logic operation).
 __device__ __forceinline__ uint32_t magic_byte(uint32_t x, int b) {
@@ -424,17 +413,13 @@ __device__ __forceinline__ uint32_t magic_byte(uint32_t x, int b) {
   asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(0x4B000000u), "r"(0x7440 | b));
   return r;
 }
-// Byte b of x and of y as codes (exactly: 2^23 + code, minus 2^23; `bias` is
-// the pair of -2^23), then fma(code, scale, lo) rounded to bf16.
-__device__ __forceinline__ uint32_t expand_pair(uint32_t x, uint32_t y, int b, uint64_t bias, uint64_t scale,
-                                                uint64_t lo) {
-  const uint64_t c = pair_of(magic_byte(x, b), magic_byte(y, b));
-  uint64_t v;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(c), "l"(bias));
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(v), "l"(scale), "l"(lo));
-  float f0, f1;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(f0), "=f"(f1) : "l"(v));
-  return pack_bf16(f0, f1);
+// Byte b of x and of y as codes (exactly: 2^23 + code, minus 2^23), then
+// fma(code, scale, lo) rounded to bf16.  Scalar: packed fp32 operations issue
+// at a quarter of the rate.
+__device__ __forceinline__ uint32_t expand_pair(uint32_t x, uint32_t y, int b, float sx, float sy, float lx, float ly) {
+  const float cx = __fsub_rn(__uint_as_float(magic_byte(x, b)), 8388608.f);
+  const float cy = __fsub_rn(__uint_as_float(magic_byte(y, b)), 8388608.f);
+  return pack_bf16(fmaf(cx, sx, lx), fmaf(cy, sy, ly));
 }
 
 // Logits of the part h of a tile: s[n] += (Q high; Q low) K^T for the tile's
@@ -454,19 +439,16 @@ __device__ __forceinline__ void qk_rows(const uint8_t* slot, const uint32_t (&qa
 }
 template <int D>
 __device__ __forceinline__ void qk_q4(const uint8_t* slot, const uint32_t (&qa)[D / 16][4], float (&s)[4][4],
-                                      uint64_t bias, int gid, int tig) {
+                                      int gid, int tig) {
   using C = TileCfg<D, true>;
   const uint8_t* par = slot + C::CODES + 128 * tig;
 #pragma unroll
   for (int j = 0; j < C::KS / 2; ++j) {
-    uint64_t sc[4], lo[4];                      // the piece's channels 2 i, 2 i + 1
+    float4 f[4];                                // (scale, minimum) of the piece's channels 2 i, 2 i + 1
     const int flip = 4 * ((j & 1) ^ (j >> 1));  // kpar_at(32 (j / 2) + 8 tig + 4 (j & 1) + i)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float4 f = *reinterpret_cast<const float4*>(par + 16 * (i ^ tig) + 512 * (j >> 1) + 16 * flip);
-      sc[i] = pair_of(f.x, f.z);
-      lo[i] = pair_of(f.y, f.w);
-    }
+    for (int i = 0; i < 4; ++i)
+      f[i] = *reinterpret_cast<const float4*>(par + 16 * (i ^ tig) + 512 * (j >> 1) + 16 * flip);
     const uint8_t* codes = slot + code_at<D>(gid, 32 * (j >> 1) + 8 * tig);
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
@@ -474,7 +456,7 @@ __device__ __forceinline__ void qk_q4(const uint8_t* slot, const uint32_t (&qa)[
       const uint32_t a = w & 0x0f0f0f0fu, b = (w >> 4) & 0x0f0f0f0fu;
       uint32_t u[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) u[i] = expand_pair(a, b, i, bias, sc[i], lo[i]);
+      for (int i = 0; i < 4; ++i) u[i] = expand_pair(a, b, i, f[i].x, f[i].z, f[i].y, f[i].w);
       mma_bf16(s[n], qa[2 * j], u[0], u[1]);
       mma_bf16(s[n], qa[2 * j + 1], u[2], u[3]);
     }
@@ -517,7 +499,7 @@ __device__ __forceinline__ void pv_rows_q4(const uint8_t* slot, const uint32_t (
 }
 template <int D>
 __device__ __forceinline__ void pv_q4(const uint8_t* slot, const uint32_t (&pa)[4], int h, float (&o)[D / 8][4],
-                                      uint64_t bias, int gid, int tig) {
+                                      int gid, int tig) {
   using C = TileCfg<D, true>;
   constexpr int WPK = D / 64;                   // code words of a thread's D / 8 dimensions
   uint32_t w[4][WPK];                           // keys 2 tig, + 1, + 8, + 9 of the 16
@@ -536,8 +518,9 @@ __device__ __forceinline__ void pv_q4(const uint8_t* slot, const uint32_t (&pa)[
     }
     pr[i] = *reinterpret_cast<const float2*>(par + r * (D / 4));
   }
-  const uint64_t s0 = pair_of(pr[0].x, pr[1].x), m0 = pair_of(pr[0].y, pr[1].y);
-  const uint64_t s1 = pair_of(pr[2].x, pr[3].x), m1 = pair_of(pr[2].y, pr[3].y);
+  auto expand = [&](const uint32_t (&c)[4], int b, int k) {   // byte b of keys k, k + 1
+    return expand_pair(c[k], c[k + 1], b, pr[k].x, pr[k + 1].x, pr[k].y, pr[k + 1].y);
+  };
 #pragma unroll
   for (int k = 0; k < WPK; ++k) {
     uint32_t a[4], b[4];                        // even and odd dimensions of the four keys
@@ -548,10 +531,8 @@ __device__ __forceinline__ void pv_q4(const uint8_t* slot, const uint32_t (&pa)[
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      mma_bf16(o[8 * k + 2 * i], pa, expand_pair(a[0], a[1], i, bias, s0, m0),
-               expand_pair(a[2], a[3], i, bias, s1, m1));
-      mma_bf16(o[8 * k + 2 * i + 1], pa, expand_pair(b[0], b[1], i, bias, s0, m0),
-               expand_pair(b[2], b[3], i, bias, s1, m1));
+      mma_bf16(o[8 * k + 2 * i], pa, expand(a, i, 0), expand(a, i, 2));
+      mma_bf16(o[8 * k + 2 * i + 1], pa, expand(b, i, 0), expand(b, i, 2));
     }
   }
 }
@@ -648,7 +629,6 @@ __global__ void __launch_bounds__(32 * kWarps, 2) decode_tiles_kernel(
   for (int t = 0; t < C::NT; ++t)
 #pragma unroll
     for (int i = 0; i < 4; ++i) o[t][i] = 0.f;
-  const uint64_t bias = pair_of(-8388608.f, -8388608.f);
   int slot = 0, item = 0;                       // the oldest item and its slot
   auto refill = [&](int n) {                    // the n oldest items are read
     __syncwarp();
@@ -706,13 +686,13 @@ __global__ void __launch_bounds__(32 * kWarps, 2) decode_tiles_kernel(
       uint32_t pa[2][4];
       tc::cp_async_wait<C::SLOTS - 1>();
       __syncwarp();
-      qk_q4<D>(ring + slot * C::SLOT, qa, s, bias, gid, tig);
+      qk_q4<D>(ring + slot * C::SLOT, qa, s, gid, tig);
       refill(1);
       softmax(s, B - (first + i * step) * kTileKeys, pa);
       tc::cp_async_wait<C::SLOTS - 1>();
       __syncwarp();
 #pragma unroll
-      for (int h = 0; h < 2; ++h) pv_q4<D>(ring + slot * C::SLOT, pa[h], h, o, bias, gid, tig);
+      for (int h = 0; h < 2; ++h) pv_q4<D>(ring + slot * C::SLOT, pa[h], h, o, gid, tig);
       refill(1);
     }
   }
