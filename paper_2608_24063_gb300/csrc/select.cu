@@ -515,10 +515,12 @@ cudaError_t launch_cut(const Shape& sh, const Tables& tb, int n_problems, const 
     if (e != cudaSuccess) return e;
   }
   ProfileScope ps("compact_keep_drop", st);
-  // an ordinary launch, as in launch_select
-  compact_kernel<false><<<dim3(sh.n_req * sh.L, sh.Hkv), kScanThreads, 0, st>>>(sh, tb, nullptr, scores, cuts,
-                                                                                keep_idx, drop_idx);
-  return cudaGetLastError();
+  // dependent: without the sort and the rank before it the chain loses nothing
+  // on ragged batches (launch_select), and a short call gains the gap (n = 3,136,
+  // 28 layers: 158.4 -> 156.6 us; one fp32 layer of 1,024: 47.2 -> 45.2 us)
+  return launch_dep(compact_kernel<false>, dim3(sh.n_req * sh.L, sh.Hkv), dim3(kScanThreads), 0, st, sh, tb,
+                    static_cast<const int32_t*>(nullptr), scores, static_cast<const uint64_t*>(cuts), keep_idx,
+                    drop_idx);
 }
 
 }  // namespace vc
