@@ -5,6 +5,7 @@
 
 #include <atomic>
 
+#include "score_shares.h"
 #include "vc_common.cuh"
 
 namespace vc {
@@ -72,11 +73,6 @@ cudaError_t launch_score_simt(int dtype, const void* Qw, const void* K, const Sh
 // Eq. (token_score) on tcgen05 tensor cores (bf16, d = 128): lse pass (skipped when
 // lse_nat != nullptr), merge of key splits, column sums.  `scratch` (nullable,
 // 16-byte aligned, overwritten) lets the column sums cut units between layers.
-struct TcReq {       // one request in the column-sum pass
-  int units2;        // key-tile units (Hkv * tiles, 0 when no layer is scored)
-  int layers;        // layers scored
-  int C, cw;         // chunks of a layer's rows, rows per chunk
-};
 struct TcPlan {
   int units1;        // units of the lse pass (sum over requests of L*Hkv*nrb*S)
   int units2;        // units of the column-sum pass (sum of Hkv*tiles)

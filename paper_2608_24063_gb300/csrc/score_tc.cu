@@ -110,7 +110,6 @@ constexpr uint32_t kPairKeys = 256;             // keys per pass-1 tile (both CT
 constexpr int kStagesPair = 4;                  // K ring of pass 1 (per CTA: 32 KB a stage)
 constexpr int kSlots1 = 2;                      // tensor-memory slots of 256 columns
 constexpr int kMaxUnits1 = 256;                 // units per pair and launch (descriptor table)
-constexpr int kMaxPairs2 = 128;                 // pass 2: shares per launch
 
 struct Unit1 {                                  // one unit as this CTA sees it
   int32_t qrow, krow;                           // Qw row of this CTA's first window row; K row of its first key
@@ -169,8 +168,11 @@ score_lse_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   }
   // the plan tables come from the kernel just before this one
   dep_wait();
+  if (split_counts && blockIdx.x == 0) {       // pass 2's counts, before it can be scheduled
+    if (threadIdx.x < 2 * kMaxPairs2) split_counts[threadIdx.x] = 0;
+    __syncthreads();
+  }
   if (threadIdx.x == 0) dep_launch();
-  if (split_counts && blockIdx.x == 0 && threadIdx.x < 2 * kMaxPairs2) split_counts[threadIdx.x] = 0;   // for pass 2
   // this pair's units: positions of the longest-first order [u_lo, u_lo + u_cnt)
   // dealt to the pairs back and forth
   const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
@@ -527,24 +529,12 @@ __device__ __forceinline__ float colsum_group(uint32_t col0, const float* nl_col
 }
 constexpr int kQStagesPair = 4;                 // Q ring of pass 2 (per CTA: 32 KB + 1 KB a stage)
 
-constexpr int kMaxSegs = 256;                   // segments per pair (descriptor table)
 // Units per resident pair up to which a launch is cut into shares: the last
 // wave then wastes up to a quarter of the time.  Pairs that start inside
 // different layers draw the window rows from the L2 at different times, which
 // costs 10 to 20% a chunk: with 13 (72B shape) or 18 units a pair (ragged
 // batch of eight) shares took 4,357 against 4,288 us and 1,375 against 1,222.
 constexpr int kShareUnits = 4;
-
-// Share p covers (unit, layer) positions from (unit[p], layer[p]) up to
-// (unit[p + 1], layer[p + 1]).  Split units are numbered by unit where there are no
-// more units than shares, else by the first cut inside them.
-// whole: pair p takes unit p and the tables are not used.
-struct Shares {
-  int32_t whole;
-  int32_t by_unit;
-  int32_t unit[kMaxPairs2 + 1];
-  int16_t layer[kMaxPairs2 + 1];
-};
 
 struct Seg2 {                                   // layers [l0, l1) of one unit as this CTA sees it
   int64_t score;                                // first score of this CTA's keys (layer 0)
@@ -601,20 +591,21 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   const bool per_layer = sh.rank_mode == VC_RANK_PER_LAYER;
 
   // this pair's segments
-  const bool whole = shares.whole != 0;
-  const int u0 = whole ? pair : shares.unit[pair], u1 = whole ? pair + 1 : shares.unit[pair + 1];
-  const int nsegs = whole ? 1 : min(kMaxSegs, u1 - u0 + (shares.layer[pair + 1] > 0 ? 1 : 0));
+  const int nsegs = min(kMaxSegs, share_segments(shares, pair));
   for (int i = threadIdx.x; i < nsegs; i += kThreads) {
-    const int unit = u0 + i;
+    const int unit = (shares.whole ? pair : shares.unit[pair]) + i;
     const int r = upper_index(tb.unit0_tc2, sh.n_req, (int32_t)unit);
     const Req& rq = tb.req[r];
+    const ShareSegment part = share_segment(shares, npairs, pair, i, rq.Ls);
     const int u = unit - tb.unit0_tc2[r];
     const int g = u / rq.tiles, kt = u % rq.tiles;
     const int key0 = kt * (int)kPairKeys + (int)rank * (int)kTile;
     Seg2 d;
     d.Ls = (int16_t)rq.Ls;
-    d.l0 = !whole && i == 0 ? shares.layer[pair] : 0;
-    d.l1 = !whole && unit == u1 ? shares.layer[pair + 1] : d.Ls;
+    d.l0 = (int16_t)part.l0;
+    d.l1 = (int16_t)part.l1;
+    d.slot = (int16_t)part.slot;
+    d.parts = (int16_t)part.parts;
     d.C = rq.C;
     d.cw = rq.cw;
     d.keys = rq.n - key0;
@@ -626,16 +617,6 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     d.kstep = sh.Hkv * rq.n;
     d.qrow = (int)(rq.q_off / 128 + (int64_t)g * sh.G * rq.W) + (int)rank * (rq.cw >> 1);
     d.qstep = sh.Hq * rq.W;
-    // a unit cut by shares a ... b - 1 (their first positions lie inside it)
-    d.slot = 0;
-    d.parts = 1;
-    if (d.l0 > 0 || d.l1 < d.Ls) {
-      int a = i == 0 && d.l0 > 0 ? pair : pair + 1, b = pair + 1;
-      while (a > 1 && shares.unit[a - 1] == unit && shares.layer[a - 1] > 0) --a;
-      while (b < npairs && shares.unit[b] == unit && shares.layer[b] > 0) ++b;
-      d.slot = (int16_t)(shares.by_unit ? unit : a);
-      d.parts = (int16_t)(b - a + 1);
-    }
     sm.seg[i] = d;
   }
   if (threadIdx.x == 0) {
@@ -766,6 +747,10 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       __syncwarp();
     }
     // ---- column sums: one thread per key (= TMEM lane)
+    // Every consumer is ordered behind the kernel before this one, also where it
+    // has no chunk whose normalisers it would wait for: split units' sums and
+    // counts go to memory that kernel may be clearing.
+    dep_wait();
     const int wg = warp >> 2;
     const int key = ((warp & 3) << 5) + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) << 5) << 16;
@@ -946,51 +931,6 @@ bool make_rows_map(CUtensorMap* m, const void* base, uint64_t rows) {
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The (unit, layer) sequence of pass 2 in equal shares of work for `pairs`
-// pairs.  Work of a layer is its rows, with 16 a chunk for what a chunk costs
-// beside them; a cut within two layers of a unit's end moves there.  False
-// when a share would have more segments than the descriptor table holds
-// (units of very unequal work).
-bool plan_shares(const TcPlan& tp, int pairs, Shares* out) {
-  int64_t total = 0;
-  auto layer_work = [](const TcReq& q) { return (int64_t)q.C * (q.cw + 16); };
-  for (int r = 0; r < tp.n_req; ++r) total += (int64_t)tp.req[r].units2 * tp.req[r].layers * layer_work(tp.req[r]);
-  out->whole = 0;
-  out->by_unit = tp.units2 <= pairs;
-  int r = 0;
-  int64_t before = 0, unit0 = 0;               // work and units of the requests before r
-  int64_t pu = 0, pl = 0;                      // previous cut
-  for (int p = 0; p <= pairs; ++p) {
-    int64_t cu = tp.units2, cl = 0;
-    if (p < pairs) {
-      const int64_t want = total / pairs * p + total % pairs * p / pairs;
-      for (; r + 1 < tp.n_req; ++r) {
-        const int64_t all = (int64_t)tp.req[r].units2 * tp.req[r].layers * layer_work(tp.req[r]);
-        if (before + all > want) break;
-        before += all;
-        unit0 += tp.req[r].units2;
-      }
-      const TcReq& q = tp.req[r];
-      const int64_t work = layer_work(q), layers = std::max(q.layers, 1);
-      const int64_t layer = (want - before + work / 2) / work;   // of the request, nearest
-      cu = unit0 + layer / layers;
-      cl = layer % layers;
-      if (cl <= 2 || cl >= layers - 2) {
-        if (2 * cl >= layers) ++cu;
-        cl = 0;
-      }
-      if (cu >= tp.units2) { cu = tp.units2; cl = 0; }
-      if (cu < pu || (cu == pu && cl < pl)) { cu = pu; cl = pl; }
-    }
-    out->unit[p] = (int32_t)cu;
-    out->layer[p] = (int16_t)cl;
-    if (p > 0 && cu - pu + 1 > kMaxSegs) return false;
-    pu = cu;
-    pl = cl;
-  }
-  return true;
-}
-
 }  // namespace
 
 int score_tc_max_splits() { return 4; }
@@ -1035,7 +975,7 @@ cudaError_t launch_score_tc(const void* Qw, const void* K, const Shape& sh, cons
                      scratch_bytes >= kSplitCountBytes + sizeof(float) * 2 * kPairKeys * (size_t)sh.L *
                                                              (size_t)std::min(tp.units2, pairs2);
   Shares shares;
-  if (!(split || per_layer) || tp.units2 > (int64_t)kShareUnits * pairs2 || !plan_shares(tp, pairs2, &shares)) {
+  if (!(split || per_layer) || tp.units2 > (int64_t)kShareUnits * pairs2 || !plan_shares(tp.req, tp.n_req, tp.units2, pairs2, &shares)) {
     memset(&shares, 0, sizeof(shares));
     shares.whole = 1;
   }
