@@ -167,6 +167,12 @@ constexpr int kSelCap = 512;
 constexpr int kSelPool = 8192;
 constexpr int kSelCuts = 257;                // 256 layers and Nq
 constexpr int kSelHeld = 16384;              // tokens whose keys are kept in shared memory
+// Every round finishes its first open cut or narrows that cut's range to one of
+// 16,384 parts, and 48 bits of composite are gone after four: with scores that
+// stand still no search takes more rounds than this.  Scores that change under
+// it (a caller that shares a workspace between streams; past kSelHeld tokens
+// they are read again) could leave a cut's range empty and the search without an end.
+constexpr int kSelRounds = 4 * kSelCuts;
 
 struct SelSmem {
   uint32_t count[kSelBuckets];               // counts, then first positions; a collected part: top bit | its cut
@@ -257,7 +263,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) threshold_kernel(Shape sh, Tab
     sm.lo[t] = (uint64_t)kmin << 16;
     sm.hi[t] = (uint64_t)kmax << 16 | 0xffffu;
   }
-  for (int round = 0;; ++round) {
+  for (int round = 0; round < kSelRounds; ++round) {
     if (t == 0) sm.todo = kSelCuts;
     __syncthreads();
     if (t < ncut && sm.pos[t] >= 0) atomicMin(&sm.todo, t);
@@ -367,7 +373,10 @@ __global__ void __launch_bounds__(kSelThreads, 1) threshold_kernel(Shape sh, Tab
     }
     __syncthreads();
   }
-  if (t < ncut) cuts[(int64_t)blockIdx.x * ncut + t] = sm.lo[t];
+  if (t < ncut) {
+    if (sm.pos[t] >= 0) set_status(tb.status, VC_ERR_DEVICE_INDEX);
+    cuts[(int64_t)blockIdx.x * ncut + t] = sm.lo[t];
+  }
 }
 
 // One CTA per (request, layer, KV head); layers with B_l == 0 exit at once.
