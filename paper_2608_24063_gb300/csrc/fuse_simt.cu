@@ -7,7 +7,7 @@
 //   Empty drop set: V_out = V_k.  The CTA also copies its kept keys, K_out =
 //   K[keep] (bit-exact 16-byte pieces).
 // R is 4, or 1 where that would leave SMs idle (one layer of 1,024 fp32 tokens:
-// 32 CTAs); rows in shared memory are read 16 bytes at a time.  Measured on
+// 32 CTAs of 32 rows); rows in shared memory are read 16 bytes at a time.  Measured on
 // that problem, with the key copy (a kernel of its own before): 23.0 -> 12.7 us.
 #include "vc_common.cuh"
 #include "kernels.h"
@@ -191,9 +191,12 @@ template <typename T, int D>
 cudaError_t launch_fuse_t(const void* K, const void* V, const Shape& sh, const Tables& tb, const int32_t* keep_idx,
                           const int32_t* drop_idx, float mu, float tau, void* K_out, void* V_out, int units,
                           cudaStream_t st) {
-  // fewer CTAs of 32 rows than two per SM: 8 rows each
-  return units < 304 ? launch_fuse_r<T, D, 1>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st)
-                     : launch_fuse_r<T, D, 4>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st);
+  // 8 rows a CTA while all of those fit at once, five an SM at d = 128: fewer of
+  // them leave SMs idle, more read the dropped rows too often (us, 32 | 8 rows:
+  // 114 units 52 | 43, 171 54 | 39, 238 127 | 228, 342 48 | 61)
+  if (4 * (int64_t)units <= 5 * (int64_t)sm_count())
+    return launch_fuse_r<T, D, 1>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st);
+  return launch_fuse_r<T, D, 4>(K, V, sh, tb, keep_idx, drop_idx, mu, tau, K_out, V_out, units, st);
 }
 
 }  // namespace

@@ -65,6 +65,9 @@ int score_rows_per_tile_simt();
 int score_keys_per_tile_simt();
 int fuse_rows_per_tile_simt();
 
+// SMs of the current device.
+int sm_count();
+
 // Eq. (token_score) on CUDA cores: lse pass (skipped when lse_nat != nullptr) + column sums.
 cudaError_t launch_score_simt(int dtype, const void* Qw, const void* K, const Shape& sh,
                               const Tables& tb, int units_lse, int units_col, float* lse,

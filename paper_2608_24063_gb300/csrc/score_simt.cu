@@ -10,11 +10,21 @@
 //
 // Few, short problems (one layer of 1,024 fp32 tokens) are bound by latency: a
 // CTA then takes a row a warp (pass 1) or a key a lane (pass 2) instead of four
-// and two, so that more of them share the work; every row's and key's
-// arithmetic stays the same.  Tiles are read from shared memory 16 bytes at a
-// time (rows padded to 4 words mod 32, free of bank conflicts) and the next
-// tile loads while the current one is used.  Measured on that problem (event
-// times, before -> now): pass 1 44.9 -> 22.3 us, pass 2 11.7 -> 9.1 us.
+// and two, so that more of them share the work, and the next tile loads into
+// registers while the current one is used.  Larger problems are bound by the
+// fma and shared-memory pipes with several CTAs an SM: there the registers that
+// hold a tile would cost CTAs (24 layers of 12,544 bf16 tokens, d = 64: pass 2
+// 2,055 us with them, 1,362 without).  Every row's and key's arithmetic is the
+// same in all forms.  Tiles are read from shared memory 16 bytes at a time (rows
+// padded to 4 words mod 32, free of bank conflicts).
+// Measured on the 1,024-token layer (event times, before -> now): pass 1 44.9 ->
+// 22.3 us, pass 2 11.7 -> 9.1 us.  Whole calls, bf16, d = 64, 24 layers of 14 / 2
+// heads, window 64, against tiles read 4 bytes at a time by ordinary launches:
+// n = 3,136 1,268 -> 1,162 us, 12,544 3,944 -> 3,778; fp32, d = 128, 8 layers of
+// 8 / 4 heads, n = 3,136 582 -> 502.
+// The next kernel may be scheduled only once a CTA has its sums: triggered
+// at the start, its CTAs filled whichever SMs came free first (n = 3,136 of
+// the above: 1,525 us instead of 1,252).
 #include "vc_common.cuh"
 #include "kernels.h"
 #include "profile.h"
@@ -86,16 +96,16 @@ __device__ __forceinline__ const T* row_set(const T* Qw, const Req& rq, const Sh
 }
 
 // Pass 1: grid (units over (request, row tile) x 32 / (8 R), L, Hkv); R rows a warp.
-template <typename T, int D, int R>
-__global__ void __launch_bounds__(kThreads) lse_simt_kernel(const T* __restrict__ Qw,
+template <typename T, int D, int R, int BLOCKS>
+__global__ void __launch_bounds__(kThreads, BLOCKS) lse_simt_kernel(const T* __restrict__ Qw,
                                                             const T* __restrict__ K, Shape sh,
                                                             Tables tb, float* __restrict__ lse) {
   extern __shared__ float4 smem4[];
   constexpr int kBlockRows = 8 * R, kSub = kRows / kBlockRows;
+  constexpr bool kAhead = R == 1;                              // next tile loads under the current one
   float* qs = reinterpret_cast<float*>(smem4);                 // [kBlockRows][D + 4]
-  float* ks = qs + kBlockRows * (D + 4);                       // [2][kKeys][D + 4]
+  float* ks = qs + kBlockRows * (D + 4);                       // [kAhead ? 2 : 1][kKeys][D + 4]
   dep_wait();                                                  // the plan tables
-  if (threadIdx.x == 0) dep_launch();
   const int unit = blockIdx.x / kSub;
   const int r = upper_index(tb.unit0_lse, sh.n_req, (int32_t)unit);
   const Req& rq = tb.req[r];
@@ -112,18 +122,26 @@ __global__ void __launch_bounds__(kThreads) lse_simt_kernel(const T* __restrict_
   auto load_keys = [&](int v0) {
     kp.load([&](int i) { return v0 + i < n ? Kl + (int64_t)(v0 + i) * D : nullptr; });
   };
-  load_keys(0);
   qp.store(qs);
-  kp.store(ks);
-  __syncthreads();
+  if (kAhead) {
+    load_keys(0);
+    kp.store(ks);
+    __syncthreads();
+  }
   float m[R], z[R];
 #pragma unroll
   for (int a = 0; a < R; ++a) { m[a] = -INFINITY; z[a] = 0.f; }
 
   int buf = 0;
-  for (int v0 = 0; v0 < n; v0 += kKeys, buf ^= 1) {
+  for (int v0 = 0; v0 < n; v0 += kKeys, buf ^= kAhead ? 1 : 0) {
     const bool more = v0 + kKeys < n;
-    if (more) load_keys(v0 + kKeys);
+    if (!kAhead) {
+      load_keys(v0);
+      kp.store(ks);
+      __syncthreads();
+    } else if (more) {
+      load_keys(v0 + kKeys);
+    }
     float acc[R][2];
     tile_dots<D, R, 2>(acc, qs + R * warp * (D + 4), ks + (buf * kKeys + lane) * (D + 4));
     const bool ok0 = v0 + lane < n, ok1 = v0 + lane + 32 < n;
@@ -137,9 +155,10 @@ __global__ void __launch_bounds__(kThreads) lse_simt_kernel(const T* __restrict_
         m[a] = mn;
       }
     }
-    if (more) kp.store(ks + (buf ^ 1) * kKeys * (D + 4));
+    if (kAhead && more) kp.store(ks + (buf ^ 1) * kKeys * (D + 4));
     __syncthreads();
   }
+  if (threadIdx.x == 0) dep_launch();
   // merge the 32 lanes' partial (max, sum) of each row
 #pragma unroll
   for (int a = 0; a < R; ++a) {
@@ -173,12 +192,13 @@ __global__ void __launch_bounds__(kThreads) colsum_simt_kernel(const T* __restri
                                                                float* __restrict__ scores) {
   extern __shared__ float4 smem4[];
   constexpr int kBlockKeys = 32 * KPL, kSub = kKeys / kBlockKeys;
-  float* qs = reinterpret_cast<float*>(smem4);                 // [2][kRows][D + 4]
-  float* ks = qs + 2 * kRows * (D + 4);                        // [kBlockKeys][D + 4]
-  float* ls = ks + kBlockKeys * (D + 4);                       // [2][kRows]
-  float (*red)[kBlockKeys] = reinterpret_cast<float (*)[kBlockKeys]>(ls + 2 * kRows);
+  constexpr bool kAhead = KPL == 1;                            // next rows and keys load under the current ones
+  constexpr int kBufs = kAhead ? 2 : 1;
+  float* qs = reinterpret_cast<float*>(smem4);                 // [kBufs][kRows][D + 4]
+  float* ks = qs + kBufs * kRows * (D + 4);                    // [kBlockKeys][D + 4]
+  float* ls = ks + kBlockKeys * (D + 4);                       // [kBufs][kRows]
+  float (*red)[kBlockKeys] = reinterpret_cast<float (*)[kBlockKeys]>(ls + kBufs * kRows);
   dep_wait();                                                  // the tables and pass 1's normalisers
-  if (threadIdx.x == 0) dep_launch();
   const int unit = blockIdx.x / kSub;
   const int r = upper_index(tb.unit0_col, sh.n_req, (int32_t)unit);
   const Req& rq = tb.req[r];
@@ -214,21 +234,28 @@ __global__ void __launch_bounds__(kThreads) colsum_simt_kernel(const T* __restri
     const T* Kl = K + rq.kv_off + (int64_t)(l * sh.Hkv + g) * n * D;
     kp.load([&](int i) { return v0 + i < n ? Kl + (int64_t)(v0 + i) * D : nullptr; });
   };
-  load_rows(0);
-  load_keys(0);
-  store_rows(0);
+  if (kAhead) {
+    load_rows(0);
+    load_keys(0);
+    store_rows(0);
+  }
   Kahan tot[KPL], lay[KPL];
 #pragma unroll
   for (int b = 0; b < KPL; ++b) { tot[b].init(); lay[b].init(); }
   for (int step = 0; step < steps; ++step) {
-    const int l = step / tiles, tile = step % tiles, buf = step & 1;
+    const int l = step / tiles, tile = step % tiles, buf = kAhead ? step & 1 : 0;
+    if (!kAhead) {
+      load_rows(step);
+      store_rows(0);
+    }
     if (tile == 0) {
+      if (!kAhead) load_keys(l);
       kp.store(ks);                              // the layer's keys (their readers are past the last barrier)
 #pragma unroll
       for (int b = 0; b < KPL; ++b) lay[b].init();
     }
     __syncthreads();
-    if (step + 1 < steps) {
+    if (kAhead && step + 1 < steps) {
       load_rows(step + 1);
       if (tile == tiles - 1) load_keys(l + 1);
     }
@@ -240,8 +267,11 @@ __global__ void __launch_bounds__(kThreads) colsum_simt_kernel(const T* __restri
 #pragma unroll
       for (int b = 0; b < KPL; ++b) lay[b].add(exp2f(fmaf(acc[a][b], sh.scale_log2, -lz)));
     }
-    if (step + 1 < steps) store_rows(buf ^ 1);
-    if (tile < tiles - 1) continue;
+    if (kAhead && step + 1 < steps) store_rows(buf ^ 1);
+    if (tile < tiles - 1) {
+      if (!kAhead) __syncthreads();              // the rows are read: the next ones may come
+      continue;
+    }
     if (sh.rank_mode == VC_RANK_PER_LAYER) {
 #pragma unroll
       for (int b = 0; b < KPL; ++b) red[warp][lane + 32 * b] = lay[b].s;
@@ -257,6 +287,7 @@ __global__ void __launch_bounds__(kThreads) colsum_simt_kernel(const T* __restri
     }
     __syncthreads();                             // keys (and partial sums) read: the next layer's may come
   }
+  if (threadIdx.x == 0) dep_launch();
   if (sh.rank_mode != VC_RANK_PER_LAYER) {
 #pragma unroll
     for (int b = 0; b < KPL; ++b) red[warp][lane + 32 * b] = tot[b].s;
@@ -269,25 +300,23 @@ __global__ void __launch_bounds__(kThreads) colsum_simt_kernel(const T* __restri
   }
 }
 
-// Below this many CTAs of the larger tiles the smaller ones are used: they
-// read shared memory more often per product but leave fewer SMs idle.
-constexpr int64_t kFewBlocks = 304;
-
-template <typename T, int D, int R>
+template <typename T, int D, int R, int BLOCKS>
 cudaError_t launch_lse(const T* q, const T* k, const Shape& sh, const Tables& tb, int units, float* lse,
                        cudaStream_t st) {
-  const size_t smem = sizeof(float) * (8 * R + 2 * kKeys) * (D + 4);
-  cudaError_t e = cudaFuncSetAttribute(lse_simt_kernel<T, D, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem = sizeof(float) * (8 * R + (R == 1 ? 2 : 1) * kKeys) * (D + 4);
+  cudaError_t e = cudaFuncSetAttribute(lse_simt_kernel<T, D, R, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
   if (e != cudaSuccess) return e;
   ProfileScope ps("score_lse_simt", st);
-  return launch_dep(lse_simt_kernel<T, D, R>, dim3(units * (kRows / (8 * R)), sh.L, sh.Hkv), dim3(kThreads), smem, st, q,
-                    k, sh, tb, lse);
+  return launch_dep(lse_simt_kernel<T, D, R, BLOCKS>, dim3(units * (kRows / (8 * R)), sh.L, sh.Hkv), dim3(kThreads),
+                    smem, st, q, k, sh, tb, lse);
 }
 
 template <typename T, int D, int KPL>
 cudaError_t launch_colsum(const T* q, const T* k, const Shape& sh, const Tables& tb, int units, const float* lse,
                           const float* lse_nat, float* scores, cudaStream_t st) {
-  const size_t smem = sizeof(float) * ((2 * kRows + 32 * KPL) * (D + 4) + 2 * kRows + 8 * 32 * KPL);
+  constexpr int kBufs = KPL == 1 ? 2 : 1;
+  const size_t smem = sizeof(float) * ((kBufs * kRows + 32 * KPL) * (D + 4) + kBufs * kRows + 8 * 32 * KPL);
   cudaError_t e = cudaFuncSetAttribute(colsum_simt_kernel<T, D, KPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
@@ -302,21 +331,42 @@ cudaError_t launch_t(const void* Qw, const void* K, const Shape& sh, const Table
                      float* scores, cudaStream_t st) {
   const T* q = static_cast<const T*>(Qw);
   const T* k = static_cast<const T*>(K);
+  // Blocks of the larger tiles.  The smaller ones read shared memory twice as
+  // often per product, so they serve only where the others leave the chip half
+  // empty.  Pass 1, four for one (us, large | small): d = 64, 16 blocks 54 | 31,
+  // 48 78 | 68, 72 99 | 86, 96 147 | 168; d = 128, 32 123 | 72, 64 204 | 206, 80
+  // 124 | 186.  Pass 2, two for one: 64 15 | 12, 76 33 | 25 (d = 128), 100 15 | 18,
+  // 152 33 | 43 (d = 128).
+  const int sms = sm_count();
+  const int64_t blocks1 = (int64_t)units_lse * sh.L * sh.Hkv, blocks2 = (int64_t)units_col * sh.Hkv;
   cudaError_t e;
   if (!lse_nat) {
-    e = (int64_t)units_lse * sh.L * sh.Hkv < kFewBlocks ? launch_lse<T, D, 1>(q, k, sh, tb, units_lse, lse, st)
-                                                        : launch_lse<T, D, 4>(q, k, sh, tb, units_lse, lse, st);
+    // d = 64, more than two blocks an SM: five fit with 48 registers (12,544 bf16
+    // tokens, 672 blocks: 1,671 -> 1,374 us; 72 blocks: 99 -> 119)
+    if (2 * blocks1 <= sms) e = launch_lse<T, D, 1, 1>(q, k, sh, tb, units_lse, lse, st);
+    else if (D == 128 || blocks1 <= 2 * sms) e = launch_lse<T, D, 4, 4>(q, k, sh, tb, units_lse, lse, st);
+    else e = launch_lse<T, D, 4, D == 128 ? 4 : 5>(q, k, sh, tb, units_lse, lse, st);
     if (e != cudaSuccess) return e;
   }
-  return (int64_t)units_col * sh.Hkv < kFewBlocks
-             ? launch_colsum<T, D, 1>(q, k, sh, tb, units_col, lse, lse_nat, scores, st)
-             : launch_colsum<T, D, 2>(q, k, sh, tb, units_col, lse, lse_nat, scores, st);
+  return 2 * blocks2 <= sms ? launch_colsum<T, D, 1>(q, k, sh, tb, units_col, lse, lse_nat, scores, st)
+                            : launch_colsum<T, D, 2>(q, k, sh, tb, units_col, lse, lse_nat, scores, st);
 }
 
 }  // namespace
 
 int score_rows_per_tile_simt() { return kRows; }
 int score_keys_per_tile_simt() { return kKeys; }
+
+int sm_count() {
+  static std::atomic<int> cached[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+  int n = cached[dev].load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
+  cached[dev].store(n, std::memory_order_relaxed);
+  return n;
+}
 
 cudaError_t launch_score_simt(int dtype, const void* Qw, const void* K, const Shape& sh,
                               const Tables& tb, int units_lse, int units_col, float* lse,
