@@ -803,8 +803,11 @@ int viscache_decode_attention_kv4(const vc_batch* batch, const vc_params* p, int
   const DecodeWs dw = decode_ws(tb.units, p->d, tb.n_req * tb.Hkv);
   const int wc = check_ws(ws, ws_bytes, dw.total);
   if (wc != VC_OK) return wc;
+  uint8_t* w = static_cast<uint8_t*>(ws);
   return cuda_status(launch_decode_kv4(tb, p->d, q, K_codes, V_codes, K_params, V_params, K_text,
-                                       V_text, out, static_cast<cudaStream_t>(stream)));
+                                       V_text, out, reinterpret_cast<float*>(w + dw.o_o),
+                                       reinterpret_cast<float2*>(w + dw.o_ml),
+                                       static_cast<cudaStream_t>(stream)));
 }
 
 int viscache_kv4_sizes(const vc_batch* batch, const vc_params* p, int64_t* rows, int64_t* key_groups) {

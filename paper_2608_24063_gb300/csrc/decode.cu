@@ -27,7 +27,9 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
+#include "decode_plan.h"
 #include "kernels.h"
 #include "profile.h"
 #include "tc_common.cuh"
@@ -290,6 +292,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_partial_kernel(
 // shared memory, and after one cluster barrier the owners finish them.  No
 // counters or partial outputs in global memory, one kernel a call, launched
 // dependently (it waits for the previous kernel before it reads anything).
+// Batches of very unequal requests (decode_plan.h) take the PARTS form: every CTA
+// takes a part of a pair's tiles and leaves its state in the workspace, and
+// decode_merge_kernel adds the parts up.
 //
 // Measured on a GB300 (28 layers as a graph, 7B shape, n = 12,544 at 19% + 512
 // text rows; before: splits of 256 keys merged through global memory): one
@@ -300,8 +305,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_partial_kernel(
 // issue (~1,650 warp instructions a tile, most of them the expansion, on two
 // warps a scheduler).
 
-constexpr int kTileKeys = 32;                  // keys per tile (one key group of the 4-bit form)
-constexpr int kWarps = 4;                      // warps per CTA
+constexpr int kWarps = kDecTileWarps;          // warps per CTA
 constexpr int kMaxCluster = 16;                // CTAs per pair
 constexpr float kRise = 8.f;                   // log2 units
 
@@ -546,25 +550,33 @@ __device__ __forceinline__ void st_cluster4(uint32_t addr, float4 v) {
                : "memory");
 }
 
-template <int D, bool Q4>
+template <int D, bool Q4, bool PARTS>
 __global__ void __launch_bounds__(32 * kWarps, 2) decode_tiles_kernel(
-    const __grid_constant__ DecodeTable tb, int cluster, const __nv_bfloat16* __restrict__ q,
+    const __grid_constant__ DecodeTable tb, int cluster_or_1, const __nv_bfloat16* __restrict__ q,
     const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __restrict__ Vc,
     const __nv_bfloat16* __restrict__ Kt, const __nv_bfloat16* __restrict__ Vt,
     const uint8_t* __restrict__ Kq, const uint8_t* __restrict__ Vq, const float* __restrict__ Kqp,
-    const float* __restrict__ Vqp, __nv_bfloat16* __restrict__ out) {
+    const float* __restrict__ Vqp, __nv_bfloat16* __restrict__ out, float* __restrict__ part_o,
+    float2* __restrict__ part_ml) {
   using C = TileCfg<D, Q4>;
   extern __shared__ __align__(128) uint8_t dsm[];
+  const int cluster = PARTS ? 1 : cluster_or_1;
   const int warp = (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gid = lane >> 2, tig = lane & 3;
   const int rank = (int)blockIdx.x % cluster, pair = (int)blockIdx.x / cluster;
-  const int r = pair / tb.Hkv, g = pair % tb.Hkv, G = tb.G;
+  // PARTS: CTA u of a request's units is part u % nsplit of its pair u / nsplit
+  const int r = PARTS ? find_req(tb, pair) : pair / tb.Hkv;
+  const int nparts = PARTS ? tb.req[r].nsplit : 1, u = PARTS ? pair - tb.req[r].unit0 : pair % tb.Hkv;
+  const int g = u / nparts, G = tb.G;
   const int B = tb.req[r].B, T = tb.req[r].T;
   const int64_t vis0 = tb.req[r].vis_row0 + (int64_t)g * B, txt0 = tb.req[r].txt_row0 + (int64_t)g * T;
   const int64_t kg0 = tb.req[r].kg0 + (int64_t)g * tb.req[r].nkg;
   const int nvt = (B + kTileKeys - 1) / kTileKeys, nt = nvt + (T + kTileKeys - 1) / kTileKeys;
-  const int first = rank * kWarps + warp, step = cluster * kWarps;
-  const int mine = nt > first ? (nt - first + step - 1) / step : 0;
+  // this CTA's tiles [lo, hi)
+  const int per = PARTS ? decode_tiles_per_part(nt, nparts) : nt;
+  const int lo = PARTS ? u % nparts * per : 0, hi = PARTS ? min(nt, lo + per) : nt;
+  const int first = lo + rank * kWarps + warp, step = cluster * kWarps;
+  const int mine = hi > first ? (hi - first + step - 1) / step : 0;
   uint8_t* ring = dsm + warp * C::RING;
   const uint32_t ring_s = tc::smem_u32(ring);
   float2* ml = reinterpret_cast<float2*>(dsm + kWarps * C::RING);            // [warp][query] (max, sum)
@@ -577,7 +589,8 @@ __global__ void __launch_bounds__(32 * kWarps, 2) decode_tiles_kernel(
 
   // Ring items, a commit group each: a tile of bf16 rows is PARTS items of K
   // rows and as many of V rows, a 4-bit tile one of each (those come first).
-  const int q4_tiles = Q4 && nvt > first ? (nvt - first + step - 1) / step : 0;
+  const int q4_end = min(nvt, hi);
+  const int q4_tiles = Q4 && q4_end > first ? (q4_end - first + step - 1) / step : 0;
   auto issue = [&](int item, int slot) {
     const uint32_t dst = ring_s + slot * C::SLOT;
     if (Q4 && item < 2 * q4_tiles) {
@@ -775,7 +788,10 @@ __global__ void __launch_bounds__(32 * kWarps, 2) decode_tiles_kernel(
 #pragma unroll
     for (int w = 0; w < kWarps; ++w)
       fold(acc, L, *reinterpret_cast<const float4*>(dsm + w * C::RING + item * 16), ml[w * kGm + jj], M);
-    if (cluster == 1) {
+    if (PARTS) {
+      *reinterpret_cast<float4*>(part_o + (int64_t)pair * kGm * D + item * 4) = acc;
+      if (d4 == 0) part_ml[(int64_t)pair * kGm + jj] = make_float2(M, L);
+    } else if (cluster == 1) {
       store(item, acc, M, L);
     } else {
       st_cluster4(tc::map_to_rank(tc::smem_u32(cout + rank * own + item % own), item / own), acc);
@@ -855,6 +871,68 @@ __global__ void __launch_bounds__(128) decode_combine_kernel(const __grid_consta
   for (int i = 0; i < EPL; ++i) dst[i] = Elem<T>::from_f(acc[i] * inv);
 }
 
+// One CTA per (request, query head): merge the parts of its KV head.  Warp w
+// sums parts w, w + 4, ... with eight parts' loads in flight; the four sums are
+// added in order.  (1,024 parts a pair took 380 us on a warp with four in flight.)
+constexpr int kMergeWarps = 4;
+template <int D>
+__global__ void __launch_bounds__(32 * kMergeWarps) decode_merge_kernel(const __grid_constant__ DecodeTable tb,
+                                                                        const float* __restrict__ part_o,
+                                                                        const float2* __restrict__ part_ml,
+                                                                        __nv_bfloat16* __restrict__ out) {
+  constexpr int EPL = D / 32;                   // output elements per lane
+  __shared__ float wmax[kMergeWarps], wsum[kMergeWarps], wo[kMergeWarps][D];
+  dep_wait();                                   // the parts' states
+  if (threadIdx.x == 0) dep_launch();
+  const int warp = (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = (int)blockIdx.x / tb.Hq, j = (int)blockIdx.x % tb.Hq, g = j / tb.G, jj = j % tb.G;
+  const int ns = tb.req[r].B + tb.req[r].T > 0 ? tb.req[r].nsplit : 0;
+  const int64_t u0 = tb.req[r].unit0 + (int64_t)g * tb.req[r].nsplit;
+  const float2* ml = part_ml + u0 * kGm + jj;
+  const float* po = part_o + (u0 * kGm + jj) * D + lane * EPL;
+  float M = -INFINITY;
+  for (int s = threadIdx.x; s < ns; s += 32 * kMergeWarps) M = fmaxf(M, ml[(int64_t)s * kGm].x);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  if (lane == 0) wmax[warp] = M;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kMergeWarps; ++w) M = fmaxf(M, wmax[w]);
+  float L = 0.f, acc[EPL] = {};
+#pragma unroll 8
+  for (int s = warp; s < ns; s += kMergeWarps) {
+    const float2 st = ml[(int64_t)s * kGm];
+    const float wt = exp2f(st.x - M);           // no part with a finite logit: NaN, as the softmax
+    L = fmaf(st.y, wt, L);
+    const float* o = po + (int64_t)s * kGm * D;
+    if constexpr (EPL == 4) {
+      const float4 v = *reinterpret_cast<const float4*>(o);
+      acc[0] = fmaf(v.x, wt, acc[0]);
+      acc[1] = fmaf(v.y, wt, acc[1]);
+      acc[EPL - 2] = fmaf(v.z, wt, acc[EPL - 2]);
+      acc[EPL - 1] = fmaf(v.w, wt, acc[EPL - 1]);
+    } else {
+      const float2 v = *reinterpret_cast<const float2*>(o);
+      acc[0] = fmaf(v.x, wt, acc[0]);
+      acc[1] = fmaf(v.y, wt, acc[1]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < EPL; ++i) wo[warp][lane * EPL + i] = acc[i];
+  if (lane == 0) wsum[warp] = L;
+  __syncthreads();
+  for (int d = threadIdx.x; d < D; d += 32 * kMergeWarps) {
+    float sum = 0.f, total = 0.f;
+#pragma unroll
+    for (int w = 0; w < kMergeWarps; ++w) {
+      sum += wo[w][d];
+      total += wsum[w];
+    }
+    const float inv = total > 0.f ? 1.f / total : 0.f;
+    out[((int64_t)r * tb.Hq + j) * D + d] = __float2bfloat16_rn(sum * inv);
+  }
+}
+
 template <typename T, int D>
 cudaError_t launch_decode_t(const DecodeTable& tb, const void* q, const void* Kc, const void* Vc,
                             const void* Kt, const void* Vt, void* out, float* part_o, float2* part_ml,
@@ -886,35 +964,9 @@ cudaError_t launch_decode_t(const DecodeTable& tb, const void* q, const void* Kc
   return cudaGetLastError();
 }
 
-// Cluster sizes decode_tiles_kernel is launched with.
-constexpr int kClusterSizes[] = {1, 2, 3, 4, 5, 6, 7, 8, 12, 16};
-constexpr int kClusterKinds = (int)(sizeof(kClusterSizes) / sizeof(int));
-
-// How many clusters of each size fit on a device at once (0: not launchable).
-struct DecodeFit {
-  int n[kClusterKinds] = {};
-};
-
-// CTAs per (request, KV head): the smallest cluster that gives every warp at
-// most one tile, or else the largest with which all pairs are on the device at
-// once (measured: one request, 137 tiles a pair, 10.4 us a layer with 4
-// CTAs, 7.0 with 8, 5.7 with 16; 16 requests 24.0 to 24.3 us with 2 or 4 CTAs
-// a pair and 28.5 with 6, which no longer fit at once).  The 4-bit kernel
-// takes the same sizes, so that its tiles are split and merged as the bf16
-// kernel's are.
-int decode_cluster(const DecodeTable& tb, const DecodeFit& fit) {
-  int tiles = 0;
-  for (int r = 0; r < tb.n_req; ++r)
-    tiles = std::max(tiles, (tb.req[r].B + kTileKeys - 1) / kTileKeys + (tb.req[r].T + kTileKeys - 1) / kTileKeys);
-  int best = 1;
-  for (int k = 1; k < kClusterKinds && best * kWarps < tiles; ++k)
-    if (fit.n[k] >= tb.n_req * tb.Hkv) best = kClusterSizes[k];
-  return best;
-}
-
-template <int D, bool Q4>
+template <int D, bool Q4, bool PARTS>
 cudaError_t prepare_decode_tiles() {
-  auto kernel = decode_tiles_kernel<D, Q4>;
+  auto kernel = decode_tiles_kernel<D, Q4, PARTS>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TileCfg<D, Q4>::SMEM);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -923,8 +975,8 @@ cudaError_t prepare_decode_tiles() {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
 }
 
-// Prepares both forms of the kernel on the current device at its first call
-// and returns what fits (the same for both: one shared-memory size).
+// Prepares the forms of the kernel on the current device at its first call
+// and returns what fits (the same for all: one shared-memory size).
 template <int D>
 cudaError_t decode_fit(DecodeFit* fit) {
   static_assert(TileCfg<D, false>::SMEM == TileCfg<D, true>::SMEM, "both forms occupy an SM alike");
@@ -937,8 +989,10 @@ cudaError_t decode_fit(DecodeFit* fit) {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> hold(guard);
   if (!known[dev]) {
-    e = prepare_decode_tiles<D, false>();
-    if (e == cudaSuccess) e = prepare_decode_tiles<D, true>();
+    e = prepare_decode_tiles<D, false, false>();
+    if (e == cudaSuccess) e = prepare_decode_tiles<D, true, false>();
+    if (e == cudaSuccess) e = prepare_decode_tiles<D, false, true>();
+    if (e == cudaSuccess) e = prepare_decode_tiles<D, true, true>();
     if (e != cudaSuccess) return e;
     for (int k = 0; k < kClusterKinds; ++k) {
       cudaLaunchAttribute at[1];
@@ -951,7 +1005,7 @@ cudaError_t decode_fit(DecodeFit* fit) {
       cfg.dynamicSmemBytes = TileCfg<D, false>::SMEM;
       cfg.attrs = at;
       cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&fits[dev].n[k], decode_tiles_kernel<D, false>, &cfg) != cudaSuccess) {
+      if (cudaOccupancyMaxActiveClusters(&fits[dev].n[k], decode_tiles_kernel<D, false, false>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         fits[dev].n[k] = 0;
       }
@@ -962,22 +1016,46 @@ cudaError_t decode_fit(DecodeFit* fit) {
   return cudaSuccess;
 }
 
+// The 4-bit form takes the same clusters and parts as the bf16 form, so that its
+// tiles are split and merged alike.
 template <int D, bool Q4>
 cudaError_t launch_decode_tiles(const DecodeTable& tb, const void* q, const void* Kc, const void* Vc,
                                 const void* Kt, const void* Vt, const uint8_t* Kq, const uint8_t* Vq,
-                                const float* Kqp, const float* Vqp, void* out, cudaStream_t st) {
+                                const float* Kqp, const float* Vqp, void* out, float* part_o, float2* part_ml,
+                                cudaStream_t st) {
   using B16 = __nv_bfloat16;
   if (tb.n_req < 1) return cudaSuccess;
   DecodeFit fit;
-  const cudaError_t e = decode_fit<D>(&fit);
+  cudaError_t e = decode_fit<D>(&fit);
   if (e != cudaSuccess) return e;
-  const int cluster = decode_cluster(tb, fit);
-  ProfileScope ps(Q4 ? "decode_attn_kv4" : "decode_attn", st);
-  return launch_dep_clusters(decode_tiles_kernel<D, Q4>, dim3((unsigned)(tb.n_req * tb.Hkv * cluster)),
-                             dim3(32 * kWarps), (size_t)TileCfg<D, Q4>::SMEM, cluster, st, tb, cluster,
-                             static_cast<const B16*>(q), static_cast<const B16*>(Kc), static_cast<const B16*>(Vc),
-                             static_cast<const B16*>(Kt), static_cast<const B16*>(Vt), Kq, Vq, Kqp, Vqp,
-                             static_cast<B16*>(out));
+  int64_t tiles[kDecodeMaxReq];
+  for (int r = 0; r < tb.n_req; ++r) tiles[r] = decode_tiles(tb.req[r].B, tb.req[r].T);
+  const DecodePlan plan = plan_decode(tiles, tb.n_req, tb.Hkv, fit);
+  auto launch = [&](auto in_parts, const DecodeTable& table, int ctas) {
+    ProfileScope ps(Q4 ? "decode_attn_kv4" : "decode_attn", st);
+    return launch_dep_clusters(decode_tiles_kernel<D, Q4, decltype(in_parts)::value>, dim3((unsigned)ctas),
+                               dim3(32 * kWarps), (size_t)TileCfg<D, Q4>::SMEM, plan.cluster, st, table, plan.cluster,
+                               static_cast<const B16*>(q), static_cast<const B16*>(Kc), static_cast<const B16*>(Vc),
+                               static_cast<const B16*>(Kt), static_cast<const B16*>(Vt), Kq, Vq, Kqp, Vqp,
+                               static_cast<B16*>(out), part_o, part_ml);
+  };
+  if (plan.part_tiles == 0)
+    return launch(std::false_type{}, tb, tb.n_req * tb.Hkv * plan.cluster);
+  // the table's units become the parts: one for every kPartMin * kWarps tiles at
+  // most, so never more than the 256-key splits the workspace is sized for
+  static_assert(kPartMin * kWarps * kTileKeys >= 2 * kSplitF, "the parts' states fit the workspace of the splits");
+  DecodeTable parts = tb;
+  parts.units = 0;
+  for (int r = 0; r < tb.n_req; ++r) {
+    parts.req[r].unit0 = parts.units;
+    parts.req[r].nsplit = decode_parts(tiles[r], plan.part_tiles);
+    parts.units += tb.Hkv * parts.req[r].nsplit;
+  }
+  e = launch(std::true_type{}, parts, parts.units);
+  if (e != cudaSuccess) return e;
+  ProfileScope ps("decode_merge", st);
+  return launch_dep(decode_merge_kernel<D>, dim3((unsigned)(tb.n_req * tb.Hq)), dim3(32 * kMergeWarps), 0, st, parts,
+                    static_cast<const float*>(part_o), static_cast<const float2*>(part_ml), static_cast<B16*>(out));
 }
 
 }  // namespace
@@ -989,8 +1067,10 @@ cudaError_t launch_decode(const DecodeTable& tb, int dtype, int d, const void* q
                           float2* part_ml, cudaStream_t st) {
   if (dtype == VC_BF16) {
     if (d == 128)
-      return launch_decode_tiles<128, false>(tb, q, Kc, Vc, Kt, Vt, nullptr, nullptr, nullptr, nullptr, out, st);
-    return launch_decode_tiles<64, false>(tb, q, Kc, Vc, Kt, Vt, nullptr, nullptr, nullptr, nullptr, out, st);
+      return launch_decode_tiles<128, false>(tb, q, Kc, Vc, Kt, Vt, nullptr, nullptr, nullptr, nullptr, out, part_o,
+                                            part_ml, st);
+    return launch_decode_tiles<64, false>(tb, q, Kc, Vc, Kt, Vt, nullptr, nullptr, nullptr, nullptr, out, part_o,
+                                            part_ml, st);
   }
   if (d == 128) return launch_decode_t<float, 128>(tb, q, Kc, Vc, Kt, Vt, out, part_o, part_ml, st);
   return launch_decode_t<float, 64>(tb, q, Kc, Vc, Kt, Vt, out, part_o, part_ml, st);
@@ -998,9 +1078,10 @@ cudaError_t launch_decode(const DecodeTable& tb, int dtype, int d, const void* q
 
 cudaError_t launch_decode_kv4(const DecodeTable& tb, int d, const void* q, const uint8_t* Kq,
                               const uint8_t* Vq, const float* Kqp, const float* Vqp, const void* Kt,
-                              const void* Vt, void* out, cudaStream_t st) {
-  if (d == 128) return launch_decode_tiles<128, true>(tb, q, nullptr, nullptr, Kt, Vt, Kq, Vq, Kqp, Vqp, out, st);
-  return launch_decode_tiles<64, true>(tb, q, nullptr, nullptr, Kt, Vt, Kq, Vq, Kqp, Vqp, out, st);
+                              const void* Vt, void* out, float* part_o, float2* part_ml, cudaStream_t st) {
+  if (d == 128)
+    return launch_decode_tiles<128, true>(tb, q, nullptr, nullptr, Kt, Vt, Kq, Vq, Kqp, Vqp, out, part_o, part_ml, st);
+  return launch_decode_tiles<64, true>(tb, q, nullptr, nullptr, Kt, Vt, Kq, Vq, Kqp, Vqp, out, part_o, part_ml, st);
 }
 
 }  // namespace vc

@@ -151,7 +151,8 @@ int decode_split_keys();
 // codes and parameters; bf16 query, text rows and output).
 cudaError_t launch_decode_kv4(const DecodeTable& tb, int d, const void* q, const uint8_t* Kq,
                               const uint8_t* Vq, const float* Kqp, const float* Vqp, const void* Kt,
-                              const void* Vt, void* out, cudaStream_t st);
+                              const void* Vt, void* out, float* part_o, float2* part_ml,
+                              cudaStream_t st);
 cudaError_t launch_decode(const DecodeTable& tb, int dtype, int d, const void* q, const void* Kc,
                           const void* Vc, const void* Kt, const void* Vt, void* out, float* part_o,
                           float2* part_ml, cudaStream_t st);

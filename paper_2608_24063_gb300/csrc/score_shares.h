@@ -5,10 +5,12 @@
 
 #include <algorithm>
 
+#ifndef VC_HD
 #ifdef __CUDACC__
 #define VC_HD __host__ __device__ __forceinline__
 #else
 #define VC_HD inline
+#endif
 #endif
 
 namespace vc {
