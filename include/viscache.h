@@ -358,7 +358,11 @@ int viscache_profile_read(char* names, int name_bytes, float* total_ms, int* lau
  * PruneKV, Sec. 3.2, the visual part of layer l holds B_l rows per KV head):
  *     out[r][j] = softmax(q[r][j] . K_g^T * scale) V_g,   g = j / (Hq / Hkv),
  * over request r's B_l kept visual rows of KV head g followed by its T_r text
- * rows.  fp32 accumulation, out rounded once to the input type.
+ * rows.  fp32 accumulation, out rounded once to the input type.  The same call
+ * gives the same bits every time.  Over bf16 and 4-bit caches the order in which
+ * a request's keys are summed follows the whole batch and the device (how many
+ * thread blocks each request gets), so its last bit may differ from batch to
+ * batch; over fp32 caches it depends on the request alone.
  *
  *   batch, p      the batch and parameters prunekv_compress ran with (they fix
  *                 every B_l); 1..256 requests, Hq / Hkv <= 8
@@ -457,7 +461,7 @@ int viscache_set_kernel_path(int path);
  * only when the previous one has completed.  Results are the same either
  * way; 0 is for debugging and for timing the difference.  A call's first
  * kernel is an ordinary launch, so calls do not overlap with work queued
- * before them; the one kernel of a bf16 or 4-bit decode call is a dependent
+ * before them; the first kernel of a bf16 or 4-bit decode call is a dependent
  * launch that waits for all work before it on the stream before it reads or
  * writes any memory.  Errors: VC_ERR_INVALID_ARG unless on is 0 or 1.
  */
