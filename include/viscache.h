@@ -427,8 +427,10 @@ int viscache_decode_attention(const vc_batch* batch, const vc_params* p, int32_t
  *   K_hat, V_hat  device [rows][d] (dequantize): the reconstruction, rounded
  *                 once to the input type
  * viscache_kv4_sizes gives rows and key_groups for a batch (host only; either
- * pointer may be NULL).  Float arrays 16-byte aligned.  All buffers are
- * caller-owned; the calls are asynchronous on `stream` and need no workspace.
+ * pointer may be NULL).  Float arrays 16-byte aligned; code arrays of any
+ * alignment (16-byte aligned ones are written faster, and decode wants them).
+ * All buffers are caller-owned; the calls are asynchronous on `stream` and need
+ * no workspace.
  * Errors: VC_ERR_INVALID_ARG (shapes, NULL or misaligned pointers), the
  * planner's errors for the batch, VC_ERR_CUDA.
  */

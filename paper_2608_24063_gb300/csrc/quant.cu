@@ -138,7 +138,9 @@ __device__ __forceinline__ void load_cpt<float, 2>(const float* p, float (&v)[2]
 // whole call took 981 us when the codes' branches and a second read of the rows
 // kept the issue slots busy at 45% of the copy rate, and takes 484 us now
 // (92% of the copy rate).
-template <typename T, int D>
+// BYTES: code arrays of any alignment, stored byte by byte (a word of 2 or 16
+// bytes otherwise).
+template <typename T, int D, bool BYTES>
 __global__ void __launch_bounds__(kQuantWarps * 32) quant_kernel(
     const __grid_constant__ QuantTable tb, int units, const T* __restrict__ K, const T* __restrict__ V,
     uint8_t* __restrict__ Kc, uint8_t* __restrict__ Vc, float2* __restrict__ Kp, float2* __restrict__ Vp) {
@@ -207,10 +209,12 @@ __global__ void __launch_bounds__(kQuantWarps * 32) quant_kernel(
   uint8_t* kc = Kc + gr.row * (D / 2) + c0 / 2;
   auto store_row = [&](int i, uint32_t q) {    // the lane's CPT codes of a row
     if (i >= gr.nrows) return;
-    if constexpr (CPT == 4)
+    if constexpr (CPT == 4 && !BYTES) {
       *reinterpret_cast<uint16_t*>(kc + i * (D / 2)) = (uint16_t)q;
-    else
+    } else {
       kc[i * (D / 2)] = (uint8_t)q;
+      if constexpr (CPT == 4) kc[i * (D / 2) + 1] = (uint8_t)(q >> 8);
+    }
   };
   uint32_t seen = 0;
 #pragma unroll
@@ -318,7 +322,13 @@ __global__ void __launch_bounds__(kQuantWarps * 32) quant_kernel(
         for (int k = 0; k < 8; ++k) w[b] |= code_of(Elem<T>::to_f(src[8 * b + k]), lo, vs, vi) << (4 * k);
       }
     }
-    *reinterpret_cast<uint4*>(Vc + (gr.row + i) * (D / 2) + gv * (kGroup / 2)) = make_uint4(w[0], w[1], w[2], w[3]);
+    uint8_t* vc = Vc + (gr.row + i) * (D / 2) + gv * (kGroup / 2);
+    if constexpr (BYTES) {
+#pragma unroll
+      for (int b = 0; b < 16; ++b) vc[b] = (uint8_t)(w[b >> 2] >> (8 * (b & 3)));
+    } else {
+      *reinterpret_cast<uint4*>(vc) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
   }
 }
 
@@ -410,10 +420,11 @@ cudaError_t launch_t(const QuantTable& tb, int units, bool quantize, const void*
   const unsigned grid = (unsigned)((units + kQuantWarps - 1) / kQuantWarps);
   if (quantize) {
     ProfileScope ps("kv4_quantize", st);
-    quant_kernel<T, D><<<grid, kQuantWarps * 32, 0, st>>>(tb, units, static_cast<const T*>(K),
-                                                          static_cast<const T*>(V), Kc, Vc,
-                                                          reinterpret_cast<float2*>(Kp),
-                                                          reinterpret_cast<float2*>(Vp));
+    const bool words = reinterpret_cast<uintptr_t>(Kc) % (D == 128 ? 2 : 1) == 0 &&
+                       reinterpret_cast<uintptr_t>(Vc) % 16 == 0;
+    auto kernel = words ? quant_kernel<T, D, false> : quant_kernel<T, D, true>;
+    kernel<<<grid, kQuantWarps * 32, 0, st>>>(tb, units, static_cast<const T*>(K), static_cast<const T*>(V), Kc, Vc,
+                                              reinterpret_cast<float2*>(Kp), reinterpret_cast<float2*>(Vp));
   } else {
     ProfileScope ps("kv4_dequantize", st);
     dequant_kernel<T, D><<<grid, kQuantWarps * 32, 0, st>>>(
