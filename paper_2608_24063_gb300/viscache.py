@@ -204,6 +204,14 @@ def viscache_plan_budgets_ex(L: int, n_vis: int, rr_num: int, rr_den: int, h: in
     return B[:], nq.value, hh.value
 
 
+def _frame_counts(n_frames: Sequence[int]):
+    # by way of an array: 64 sizes take 1 us, one by one 5 us, of a call that takes 20
+    try:
+        return (ctypes.c_int32 * len(n_frames)).from_buffer(array.array("i", list(n_frames)))
+    except OverflowError:   # the library, or the check against H's rows, refuses these
+        return (ctypes.c_int32 * len(n_frames))(*n_frames)
+
+
 def viscache_scout_mmr(H: torch.Tensor, prompt: torch.Tensor, n_frames: Sequence[int], lam: float = 0.7,
                        p: Tuple[int, int] = (3, 4), with_gains: bool = True, stream=None,
                        out: Optional[Tuple[torch.Tensor, torch.Tensor, Optional[torch.Tensor]]] = None,
@@ -216,8 +224,7 @@ def viscache_scout_mmr(H: torch.Tensor, prompt: torch.Tensor, n_frames: Sequence
     """
     n_req = len(n_frames)
     D = H.shape[1]
-    # by way of an array: 64 sizes take 1 us, one by one 5 us, of a call that takes 20
-    nf = (ctypes.c_int32 * n_req).from_buffer(array.array("i", n_frames))
+    nf = _frame_counts(n_frames)
     need = lib().viscache_scout_workspace_size(n_req, nf, D)
     if need == 0:
         raise VisCacheError("viscache_scout_workspace_size", VC_ERR_INVALID_ARG)
