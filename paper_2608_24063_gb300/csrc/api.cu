@@ -53,7 +53,7 @@ struct RequestPlan {
 struct Layout {
   // inputs
   int n_req = 0, L = 0, Hq = 0, Hkv = 0, d = 0, rank_mode = VC_RANK_SHARED;
-  bool need_lse = false, need_scores = false, need_sort = false, need_drop = false, need_vs = false;
+  bool need_lse = false, need_scores = false, need_sort = false, need_cuts = false, need_drop = false, need_vs = false;
   bool prune_layers = false;   // score and rank only the layers the budgets keep (fused pass)
   // tensor-core score plan
   int S = 1;
@@ -69,13 +69,12 @@ struct Layout {
   int units_lse = 0, units_col = 0, units_fuse = 0;
   // workspace offsets
   size_t o_status = 0, o_req = 0, o_layer = 0, o_u_lse = 0, o_u_col = 0, o_u_fuse = 0,
-         o_row0 = 0, o_u_tc1 = 0, o_u_tc2 = 0, o_u_fuse_tc = 0, o_u_gather = 0, o_vs = 0, table_begin = 0, table_end = 0, o_lse = 0,
-         o_part = 0, o_lsep = 0, o_scores = 0, o_chunks = 0, o_rank = 0, o_drop = 0, total = 0;
+         o_u_tc1 = 0, o_u_tc2 = 0, o_u_fuse_tc = 0, o_u_gather = 0, o_vs = 0, table_begin = 0, table_end = 0, o_lse = 0,
+         o_part = 0, o_lsep = 0, o_scores = 0, o_chunks = 0, o_cuts = 0, o_drop = 0, total = 0;
   // host images
   std::vector<Req> req;
   std::vector<Layer> layer;
   std::vector<int32_t> u_lse, u_col, u_fuse;
-  std::vector<int64_t> row0;
 
   void build(const std::vector<RequestPlan>& plans) {
     n_req = (int)plans.size();
@@ -85,7 +84,6 @@ struct Layout {
     u_lse.assign(n_req + 1, 0);
     u_col.assign(n_req + 1, 0);
     u_fuse.assign((size_t)n_req * L + 1, 0);
-    row0.assign((size_t)n_req * L + 1, 0);
     u_tc1.assign(n_req + 1, 0);
     u_fuse_tc.assign((size_t)n_req * L + 1, 0);
     u_gather.assign((size_t)n_req * L + 1, 0);
@@ -148,7 +146,6 @@ struct Layout {
         const int32_t b = p.B.empty() ? 0 : p.B[l];
         Layer& ly = layer[rl];
         ly.B = b; ly.P = P; ly.D = b > 0 ? p.Nq - b : 0; ly.Qd = Qd;
-        row0[rl] = out_rows + (int64_t)Hkv * P;
         u_fuse[rl + 1] = u_fuse[rl] + Hkv * ((b + fuse_tile - 1) / fuse_tile);
         u_fuse_tc[rl + 1] = u_fuse_tc[rl] + Hkv * ((b + fuse_tile_tc - 1) / fuse_tile_tc);
         u_gather[rl + 1] = u_gather[rl] + Hkv * ((b + ly.D + gather_rows - 1) / gather_rows);
@@ -166,7 +163,6 @@ struct Layout {
     std::stable_sort(by_length.begin(), by_length.end(),
                      [&](int32_t a, int32_t b) { return plans[a].n > plans[b].n; });
     for (int r = 0; r < n_req; ++r) req[r].by_length = by_length[r];
-    row0[(size_t)n_req * L] = out_rows;
     lse_elems = (int64_t)L * Hq * cu_w;
     score_elems = (int64_t)per_req_problems * cu_n;
     units_lse = u_lse[n_req];
@@ -184,7 +180,6 @@ struct Layout {
     o_u_lse = a.take(sizeof(int32_t) * u_lse.size());
     o_u_col = a.take(sizeof(int32_t) * u_col.size());
     o_u_fuse = a.take(sizeof(int32_t) * u_fuse.size());
-    o_row0 = a.take(sizeof(int64_t) * row0.size());
     o_u_tc1 = a.take(sizeof(int32_t) * u_tc1.size());
     o_u_tc2 = a.take(sizeof(int32_t) * u_tc2.size());
     o_u_fuse_tc = a.take(sizeof(int32_t) * u_fuse_tc.size());
@@ -197,10 +192,10 @@ struct Layout {
       o_lsep = a.take(sizeof(float) * prows);
     }
     if (need_scores) o_scores = a.take(sizeof(float) * score_elems);
-    if (need_sort) {
-      o_chunks = a.take(sizeof(uint64_t) * kSortChunk * std::max<int64_t>(total_chunks, 1));
-      if (need_scores) o_rank = a.take(sizeof(int32_t) * score_elems);
-    }
+    if (need_sort) o_chunks = a.take(sizeof(uint64_t) * kSortChunk * std::max<int64_t>(total_chunks, 1));
+    // the fused pass's cuts: the survivors' and each layer's, or a layer's own
+    if (need_cuts)
+      o_cuts = a.take(sizeof(uint64_t) * n_req * per_req_problems * (rank_mode == VC_RANK_PER_LAYER ? 2 : L + 1));
     if (need_drop) o_drop = a.take(sizeof(int32_t) * drop_rows);
     if (need_vs) o_vs = a.take((size_t)256 * std::max<int64_t>(vs_rows, 1));
     total = a.off;
@@ -275,7 +270,6 @@ struct Layout {
     put(o_u_lse, u_lse.data(), sizeof(int32_t) * u_lse.size());
     put(o_u_col, u_col.data(), sizeof(int32_t) * u_col.size());
     put(o_u_fuse, u_fuse.data(), sizeof(int32_t) * u_fuse.size());
-    put(o_row0, row0.data(), sizeof(int64_t) * row0.size());
     put(o_u_tc1, u_tc1.data(), sizeof(int32_t) * u_tc1.size());
     put(o_u_tc2, u_tc2.data(), sizeof(int32_t) * u_tc2.size());
     put(o_u_fuse_tc, u_fuse_tc.data(), sizeof(int32_t) * u_fuse_tc.size());
@@ -289,7 +283,6 @@ struct Layout {
     t.unit0_lse = reinterpret_cast<const int32_t*>(ws + o_u_lse);
     t.unit0_col = reinterpret_cast<const int32_t*>(ws + o_u_col);
     t.unit0_fuse = reinterpret_cast<const int32_t*>(ws + o_u_fuse);
-    t.row0_out = reinterpret_cast<const int64_t*>(ws + o_row0);
     t.unit0_tc1 = reinterpret_cast<const int32_t*>(ws + o_u_tc1);
     t.unit0_tc2 = reinterpret_cast<const int32_t*>(ws + o_u_tc2);
     t.unit0_fuse_tc = reinterpret_cast<const int32_t*>(ws + o_u_fuse_tc);
@@ -454,7 +447,7 @@ int plan_batch(const vc_batch* b, const vc_params* p, std::vector<RequestPlan>* 
 Layout compress_layout(const vc_params* p, const std::vector<RequestPlan>& plans) {
   Layout lay;
   lay.L = p->L; lay.Hq = p->Hq; lay.Hkv = p->Hkv; lay.d = p->d; lay.rank_mode = p->rank_mode;
-  lay.need_lse = lay.need_scores = lay.need_sort = lay.need_drop = true;
+  lay.need_lse = lay.need_scores = lay.need_cuts = lay.need_drop = true;
   lay.need_vs = p->dtype == VC_BF16 && p->d == 128;
   lay.prune_layers = true;
   lay.build(plans);
@@ -515,12 +508,11 @@ int decode_table(const vc_params* p, const std::vector<RequestPlan>& plans, int 
 }
 
 struct DecodeWs {
-  size_t o_arr = 0, o_ml = 0, o_o = 0, total = 0;
+  size_t o_ml = 0, o_o = 0, total = 0;
 };
-DecodeWs decode_ws(int64_t units, int d, int pairs) {
+DecodeWs decode_ws(int64_t units, int d) {
   Arena a;
   DecodeWs w;
-  w.o_arr = a.take(sizeof(int32_t) * std::max(pairs, 1));
   w.o_ml = a.take(sizeof(float2) * kDecodeMaxGroup * std::max<int64_t>(units, 1));
   w.o_o = a.take(sizeof(float) * kDecodeMaxGroup * d * std::max<int64_t>(units, 1));
   w.total = a.off;
@@ -720,7 +712,7 @@ int prunekv_compress(const vc_batch* batch, const vc_params* p, const void* Qw, 
   const Shape sh = lay.shape(scale);
   const Tables tb = lay.tables(w);
   const int problems = lay.n_req * (p->rank_mode == VC_RANK_PER_LAYER ? p->L * p->Hkv : p->Hkv);
-  e = launch_cut(sh, tb, problems, scores, reinterpret_cast<uint64_t*>(w + lay.o_chunks), idx_out, drop, st);
+  e = launch_cut(sh, tb, problems, scores, reinterpret_cast<uint64_t*>(w + lay.o_cuts), idx_out, drop, st);
   if (e != cudaSuccess) return VC_ERR_CUDA;
   e = launch_fuse(p->dtype, K, V, lay, sh, tb, idx_out, drop, p->mu, p->tau, K_out, V_out, w, st);
   return cuda_status(e);
@@ -753,7 +745,7 @@ size_t viscache_decode_workspace_size(const vc_batch* batch, const vc_params* p,
     }
     units = std::max(units, u);
   }
-  return decode_ws(units, p->d, batch->n_req * p->Hkv).total;
+  return decode_ws(units, p->d).total;
 }
 
 int viscache_decode_attention(const vc_batch* batch, const vc_params* p, int32_t layer,
@@ -772,7 +764,7 @@ int viscache_decode_attention(const vc_batch* batch, const vc_params* p, int32_t
   static thread_local DecodeTable tb;
   const int tc = decode_table(p, plans, layer, n_text, &tb);
   if (tc != VC_OK) return tc;
-  const DecodeWs dw = decode_ws(tb.units, p->d, tb.n_req * tb.Hkv);
+  const DecodeWs dw = decode_ws(tb.units, p->d);
   const int wc = check_ws(ws, ws_bytes, dw.total);
   if (wc != VC_OK) return wc;
   uint8_t* w = static_cast<uint8_t*>(ws);
@@ -800,7 +792,7 @@ int viscache_decode_attention_kv4(const vc_batch* batch, const vc_params* p, int
   static thread_local DecodeTable tb;
   const int tc = decode_table(p, plans, layer, n_text, &tb);
   if (tc != VC_OK) return tc;
-  const DecodeWs dw = decode_ws(tb.units, p->d, tb.n_req * tb.Hkv);
+  const DecodeWs dw = decode_ws(tb.units, p->d);
   const int wc = check_ws(ws, ws_bytes, dw.total);
   if (wc != VC_OK) return wc;
   uint8_t* w = static_cast<uint8_t*>(ws);

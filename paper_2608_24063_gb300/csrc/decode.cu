@@ -944,7 +944,7 @@ cudaError_t launch_decode_t(const DecodeTable& tb, const void* q, const void* Kc
       cudaError_t e = cudaFuncSetAttribute(decode_partial_kernel<T, D>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
-      // the whole unified L1 as shared memory: two CTAs per SM for bf16 rows
+      // the whole unified L1 as shared memory: a d = 64 CTA is 87 KB, two an SM
       e = cudaFuncSetAttribute(decode_partial_kernel<T, D>,
                                cudaFuncAttributePreferredSharedMemoryCarveout, 100);
       if (e != cudaSuccess) return e;

@@ -112,8 +112,7 @@ cudaError_t launch_select(const Shape& sh, const Tables& tb, int n_problems, int
                           int32_t* drop_idx, cudaStream_t st);
 
 // The same lists without the ranks (the fused pass): `cuts` holds L + 1 (shared
-// ranking) or 2 (layer-specific) composites per problem; kSortChunk of them
-// always fit a problem's chunks.
+// ranking) or 2 (layer-specific) composites per problem.
 cudaError_t launch_cut(const Shape& sh, const Tables& tb, int n_problems, const float* scores, uint64_t* cuts,
                        int32_t* keep_idx, int32_t* drop_idx, cudaStream_t st);
 

@@ -54,7 +54,6 @@ struct Tables {              // device pointers into the workspace
   const int32_t* unit0_lse;  // [n_req + 1] row-tile units of the lse pass
   const int32_t* unit0_col;  // [n_req + 1] key-tile units of the column-sum pass
   const int32_t* unit0_fuse; // [n_req * L + 1] kept-row-tile units x Hkv of the fusion
-  const int64_t* row0_out;   // [n_req * L + 1] first output row of each (request, layer)
   const int32_t* unit0_tc1;  // [n_req + 1] units of the tensor-core lse pass, requests longest first
   const int32_t* unit0_tc2;  // [n_req + 1] CTAs of the tensor-core column-sum pass
   const int32_t* unit0_fuse_tc;  // [n_req * L + 1] 256-row kept tiles x Hkv (tensor-core fusion)
