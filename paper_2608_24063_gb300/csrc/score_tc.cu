@@ -747,10 +747,6 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       __syncwarp();
     }
     // ---- column sums: one thread per key (= TMEM lane)
-    // Every consumer is ordered behind the kernel before this one, also where it
-    // has no chunk whose normalisers it would wait for: split units' sums and
-    // counts go to memory that kernel may be clearing.
-    dep_wait();
     const int wg = warp >> 2;
     const int key = ((warp & 3) << 5) + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) << 5) << 16;
@@ -760,6 +756,10 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     for (int s = 0; s < nsegs; ++s) {
       const int C = sm.seg[s].C, cw = sm.seg[s].cw, l0 = sm.seg[s].l0, l1 = sm.seg[s].l1, Ls = sm.seg[s].Ls;
       const int parts = sm.seg[s].parts, slot = sm.seg[s].slot;
+      // Split units' sums and counts go to memory the kernel before this one may be
+      // clearing: every consumer is ordered behind it, also one without a chunk
+      // whose normalisers it would wait for.
+      if (!per_layer && parts > 1) dep_wait();
       const bool valid = key < sm.seg[s].keys;
       float* out = scores + sm.seg[s].score + key;
       const int nhalf = (cw + (int)kTile - 1) / (int)kTile;   // 1 or 2 halves of 128 columns
