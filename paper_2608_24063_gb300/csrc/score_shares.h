@@ -112,4 +112,12 @@ inline bool plan_shares(const TcReq* req, int n_req, int64_t units2, int pairs, 
   return true;
 }
 
+// Whether a cut lies inside a unit.  Without one, and with a pair for every unit,
+// whole units do the same with less to set up.
+inline bool cuts_a_unit(const Shares& s, int pairs) {
+  for (int p = 1; p < pairs; ++p)
+    if (s.layer[p] > 0) return true;
+  return false;
+}
+
 }  // namespace vc

@@ -36,6 +36,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "kernels.h"
 #include "profile.h"
@@ -491,7 +492,7 @@ constexpr uint32_t kChunkRows = 256;            // window rows per pass-2 chunk 
 // columns.  NP is a compile-time count so the loads and sums unroll fully.
 template <int NP>
 __device__ __forceinline__ float colsum_group(uint32_t col0, const float* nl_col, float s2, bool release,
-                                              uint64_t* tm_empty, int lane) {
+                                              uint32_t tm_empty0, int lane) {
   float x[NP][16];
   {
     uint32_t vv[NP][16];
@@ -508,7 +509,7 @@ __device__ __forceinline__ float colsum_group(uint32_t col0, const float* nl_col
   if (release) {
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(tm_empty), 0));   // slot copied out
+    if (lane == 0) mbar_arrive_cluster(tm_empty0);   // slot copied out
   }
   const float4* nl = reinterpret_cast<const float4*>(nl_col);
   float ps[8];
@@ -579,6 +580,9 @@ __device__ __forceinline__ float* split_sums(void* scratch, int slot, int Ls, in
          (((int64_t)slot * Ls + l) * 2 + wg) * kPairKeys;
 }
 
+// CUT: shares.whole is 0 (the pairs take the shares' segments); else pair p walks
+// unit p.
+template <bool CUT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                        const __grid_constant__ Shares shares, Shape sh, Tables tb, const float* __restrict__ nlse,
@@ -591,12 +595,13 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   const bool per_layer = sh.rank_mode == VC_RANK_PER_LAYER;
 
   // this pair's segments
-  const int nsegs = min(kMaxSegs, share_segments(shares, pair));
-  for (int i = threadIdx.x; i < nsegs; i += kThreads) {
-    const int unit = (shares.whole ? pair : shares.unit[pair]) + i;
+  const int nsegs = CUT ? min(kMaxSegs, share_segments(shares, pair)) : 1;
+  for (int i = (int)threadIdx.x - 32; i < nsegs; i += kThreads) {   // warp 0 sets up the barriers meanwhile
+    if (i < 0) continue;
+    const int unit = (CUT ? shares.unit[pair] : pair) + i;
     const int r = upper_index(tb.unit0_tc2, sh.n_req, (int32_t)unit);
     const Req& rq = tb.req[r];
-    const ShareSegment part = share_segment(shares, npairs, pair, i, rq.Ls);
+    const ShareSegment part = CUT ? share_segment(shares, npairs, pair, i, rq.Ls) : ShareSegment{unit, 0, rq.Ls, 0, 1};
     const int u = unit - tb.unit0_tc2[r];
     const int g = u / rq.tiles, kt = u % rq.tiles;
     const int key0 = kt * (int)kPairKeys + (int)rank * (int)kTile;
@@ -750,12 +755,14 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     const int wg = warp >> 2;
     const int key = ((warp & 3) << 5) + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) << 5) << 16;
+    const uint32_t tm_empty0 = lane == 0 ? map_to_rank(smem_u32(&sm.tm_empty[wg]), 0) : 0u;
     const float s2 = sh.scale_log2;
     int qi = 0;                                     // chunks so far
     uint32_t use = 0;                               // this warpgroup's chunks so far
     for (int s = 0; s < nsegs; ++s) {
-      const int C = sm.seg[s].C, cw = sm.seg[s].cw, l0 = sm.seg[s].l0, l1 = sm.seg[s].l1, Ls = sm.seg[s].Ls;
-      const int parts = sm.seg[s].parts, slot = sm.seg[s].slot;
+      const int C = sm.seg[s].C, cw = sm.seg[s].cw, Ls = sm.seg[s].Ls;
+      const int l0 = CUT ? sm.seg[s].l0 : 0, l1 = CUT ? sm.seg[s].l1 : Ls;
+      const int parts = CUT ? sm.seg[s].parts : 1, slot = CUT ? sm.seg[s].slot : 0;
       // Split units' sums and counts go to memory the kernel before this one may be
       // clearing: every consumer is ordered behind it, also one without a chunk
       // whose normalisers it would wait for.
@@ -793,14 +800,14 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         const float* nl = sm.nlse[qs] + hf * (int)kTile;
         const bool rel = hf == nhalf - 1;           // the slot is free after this load
         switch (np) {
-          case 8: return colsum_group<8>(col0, nl, s2, rel, &sm.tm_empty[wg], lane);
-          case 7: return colsum_group<7>(col0, nl, s2, rel, &sm.tm_empty[wg], lane);
-          case 6: return colsum_group<6>(col0, nl, s2, rel, &sm.tm_empty[wg], lane);
-          case 5: return colsum_group<5>(col0, nl, s2, rel, &sm.tm_empty[wg], lane);
-          case 4: return colsum_group<4>(col0, nl, s2, rel, &sm.tm_empty[wg], lane);
-          case 3: return colsum_group<3>(col0, nl, s2, rel, &sm.tm_empty[wg], lane);
-          case 2: return colsum_group<2>(col0, nl, s2, rel, &sm.tm_empty[wg], lane);
-          default: return colsum_group<1>(col0, nl, s2, rel, &sm.tm_empty[wg], lane);
+          case 8: return colsum_group<8>(col0, nl, s2, rel, tm_empty0, lane);
+          case 7: return colsum_group<7>(col0, nl, s2, rel, tm_empty0, lane);
+          case 6: return colsum_group<6>(col0, nl, s2, rel, tm_empty0, lane);
+          case 5: return colsum_group<5>(col0, nl, s2, rel, tm_empty0, lane);
+          case 4: return colsum_group<4>(col0, nl, s2, rel, tm_empty0, lane);
+          case 3: return colsum_group<3>(col0, nl, s2, rel, tm_empty0, lane);
+          case 2: return colsum_group<2>(col0, nl, s2, rel, tm_empty0, lane);
+          default: return colsum_group<1>(col0, nl, s2, rel, tm_empty0, lane);
         }
       };
       // one chunk (layer l) of this warpgroup: wait for its logits and
@@ -975,7 +982,9 @@ cudaError_t launch_score_tc(const void* Qw, const void* K, const Shape& sh, cons
                      scratch_bytes >= kSplitCountBytes + sizeof(float) * 2 * kPairKeys * (size_t)sh.L *
                                                              (size_t)std::min(tp.units2, pairs2);
   Shares shares;
-  if (!(split || per_layer) || tp.units2 > (int64_t)kShareUnits * pairs2 || !plan_shares(tp.req, tp.n_req, tp.units2, pairs2, &shares)) {
+  if (!(split || per_layer) || tp.units2 > (int64_t)kShareUnits * pairs2 ||
+      !plan_shares(tp.req, tp.n_req, tp.units2, pairs2, &shares) ||
+      (tp.units2 <= pairs2 && !cuts_a_unit(shares, pairs2))) {
     memset(&shares, 0, sizeof(shares));
     shares.whole = 1;
   }
@@ -1001,11 +1010,15 @@ cudaError_t launch_score_tc(const void* Qw, const void* K, const Shape& sh, cons
     if (e != cudaSuccess) return e;
   }
   const size_t smem2 = sizeof(P2Smem) + 1024;
-  e = cudaFuncSetAttribute(score_colsum_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
-  if (e != cudaSuccess) return e;
-  ProfileScope ps("score_colsum_tc", st);
-  return launch_dep(score_colsum_tc_kernel, dim3(2 * (shares.whole ? tp.units2 : pairs2)), dim3(kThreads), smem2, st,
-                    mq, mk, shares, sh, tb, static_cast<const float*>(nlse_pad), scores, scratch);
+  auto colsum = [&](auto cut, int ctas) -> cudaError_t {
+    constexpr bool kCut = decltype(cut)::value;
+    e = cudaFuncSetAttribute(score_colsum_tc_kernel<kCut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+    if (e != cudaSuccess) return e;
+    ProfileScope ps("score_colsum_tc", st);
+    return launch_dep(score_colsum_tc_kernel<kCut>, dim3(ctas), dim3(kThreads), smem2, st, mq, mk, shares, sh, tb,
+                      static_cast<const float*>(nlse_pad), scores, scratch);
+  };
+  return shares.whole ? colsum(std::false_type{}, 2 * tp.units2) : colsum(std::true_type{}, 2 * pairs2);
 }
 
 }  // namespace vc
