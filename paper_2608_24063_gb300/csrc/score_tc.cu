@@ -296,6 +296,7 @@ score_lse_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const int wg = warp >> 2;
     const int lrow = ((warp & 3) << 5) + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) << 5) << 16;
+    const uint32_t tm_empty0 = lane == 0 ? map_to_rank(smem_u32(&sm.tm_empty[wg]), 0) : 0u;
     const float s2 = sh.scale_log2;
     bool ok = true;
     uint32_t use = 0;                             // this warpgroup's tiles so far
@@ -309,13 +310,11 @@ score_lse_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       // stall the warp until the exp2 unit has worked through its queue.
       float pend = 0.f;
       for (int i = wg; ok && i < ntiles; i += 2, ++use) {
+        ok = warp_wait(&sm.tm_full[wg], use & 1, abort);
+        if (!ok) break;
+        tc_fence_after();
 #pragma unroll 1
         for (int hf = 0; hf < 2; ++hf) {
-          if (hf == 0) {
-            ok = warp_wait(&sm.tm_full[wg], use & 1, abort);
-            if (!ok) break;
-            tc_fence_after();
-          }
           const int valid = min((int)kTile, keys - i * (int)kPairKeys - hf * (int)kTile);
           const uint32_t col0 = tbase + lane_off + (uint32_t)wg * kPairKeys + (uint32_t)hf * kTile;
           float x[8][16];
@@ -334,7 +333,7 @@ score_lse_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           if (hf == 1) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.tm_empty[wg]), 0));   // slot copied out
+            if (lane == 0) mbar_arrive_cluster(tm_empty0);   // slot copied out
           }
           if (valid < (int)kTile) {                 // keys >= n (ragged last tile)
 #pragma unroll
