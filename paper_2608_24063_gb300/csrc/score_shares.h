@@ -27,9 +27,7 @@ struct TcReq {       // one request in the column-sum pass
 // Share p covers (unit, layer) positions from (unit[p], layer[p]) up to
 // (unit[p + 1], layer[p + 1]).  Split units are numbered by unit where there are no
 // more units than shares, else by the first cut inside them.
-// whole: pair p takes unit p and the tables are not used.
 struct Shares {
-  int32_t whole;
   int32_t by_unit;
   int32_t unit[kMaxPairs2 + 1];
   int16_t layer[kMaxPairs2 + 1];
@@ -38,7 +36,6 @@ struct Shares {
 // Units share p has layers of.  A share that ends where it begins has none: its
 // CTAs take no part in any unit.
 VC_HD int share_segments(const Shares& s, int p) {
-  if (s.whole) return 1;
   if (s.unit[p] == s.unit[p + 1] && s.layer[p] == s.layer[p + 1]) return 0;
   return s.unit[p + 1] - s.unit[p] + (s.layer[p + 1] > 0 ? 1 : 0);
 }
@@ -50,9 +47,9 @@ struct ShareSegment {
 };
 VC_HD ShareSegment share_segment(const Shares& s, int npairs, int p, int i, int Ls) {
   ShareSegment d;
-  d.unit = (s.whole ? p : s.unit[p]) + i;
-  d.l0 = !s.whole && i == 0 ? s.layer[p] : 0;
-  d.l1 = !s.whole && d.unit == s.unit[p + 1] ? s.layer[p + 1] : Ls;
+  d.unit = s.unit[p] + i;
+  d.l0 = i == 0 ? s.layer[p] : 0;
+  d.l1 = d.unit == s.unit[p + 1] ? s.layer[p + 1] : Ls;
   d.slot = 0;
   d.parts = 1;
   if (d.l0 > 0 || d.l1 < Ls) {
@@ -76,7 +73,6 @@ inline bool plan_shares(const TcReq* req, int n_req, int64_t units2, int pairs, 
   int64_t total = 0;
   auto layer_work = [](const TcReq& q) { return (int64_t)q.C * (q.cw + 16); };
   for (int r = 0; r < n_req; ++r) total += (int64_t)req[r].units2 * req[r].layers * layer_work(req[r]);
-  out->whole = 0;
   out->by_unit = units2 <= pairs;
   int r = 0;
   int64_t before = 0, unit0 = 0;               // work and units of the requests before r

@@ -167,6 +167,10 @@ score_lse_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     tmem_alloc_pair(&sm.tmem_base, kTmemCols);
     tmem_relinquish_pair();
   }
+  __syncwarp();
+  tc_fence_before();
+  cluster_sync();                  // barriers of both CTAs, TMEM
+  tc_fence_after();
   // the plan tables come from the kernel just before this one
   dep_wait();
   if (split_counts && blockIdx.x == 0) {       // pass 2's counts, before it can be scheduled
@@ -182,7 +186,7 @@ score_lse_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   for (int i = threadIdx.x; i < nunits; i += kThreads) {
     const int unit = u_lo + i * npairs + ((i & 1) ? npairs - 1 - pair : pair);
     const int place = upper_index(tb.unit0_tc1, sh.n_req, (int32_t)unit);
-    const Req& rq = tb.req[tb.req[place].by_length];
+    const Req& rq = tb.req[sh.n_req > 1 ? tb.req[place].by_length : 0];
     int u = unit - tb.unit0_tc1[place];
     const int split = u % S;
     u /= S;
@@ -206,10 +210,7 @@ score_lse_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                   : rq.lsep_off + ((int64_t)l * sh.Hkv + g) * d.prow;
     sm.unit[i] = d;
   }
-  __syncwarp();
-  tc_fence_before();
-  cluster_sync();                  // descriptors, barriers of both CTAs, TMEM
-  tc_fence_after();
+  __syncthreads();                 // descriptors
   const uint32_t tbase = sm.tmem_base;
   volatile int* abort = &sm.abort;
 
@@ -579,12 +580,13 @@ __device__ __forceinline__ float* split_sums(void* scratch, int slot, int Ls, in
          (((int64_t)slot * Ls + l) * 2 + wg) * kPairKeys;
 }
 
-// CUT: shares.whole is 0 (the pairs take the shares' segments); else pair p walks
-// unit p.
+// CUT: the pairs take the shares' segments; else pair p walks unit p.
+struct NoShares {};
 template <bool CUT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                       const __grid_constant__ Shares shares, Shape sh, Tables tb, const float* __restrict__ nlse,
+                       const __grid_constant__ std::conditional_t<CUT, Shares, NoShares> shares, Shape sh,
+                       Tables tb, const float* __restrict__ nlse,
                        float* __restrict__ scores, void* __restrict__ scratch) {
   extern __shared__ uint8_t smem_raw[];
   P2Smem& sm = *reinterpret_cast<P2Smem*>(align1024(smem_raw));
@@ -594,13 +596,16 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   const bool per_layer = sh.rank_mode == VC_RANK_PER_LAYER;
 
   // this pair's segments
-  const int nsegs = CUT ? min(kMaxSegs, share_segments(shares, pair)) : 1;
+  int nsegs = 1;
+  if constexpr (CUT) nsegs = min(kMaxSegs, share_segments(shares, pair));
   for (int i = (int)threadIdx.x - 32; i < nsegs; i += kThreads) {   // warp 0 sets up the barriers meanwhile
     if (i < 0) continue;
-    const int unit = (CUT ? shares.unit[pair] : pair) + i;
+    int unit = pair;
+    if constexpr (CUT) unit = shares.unit[pair] + i;
     const int r = upper_index(tb.unit0_tc2, sh.n_req, (int32_t)unit);
     const Req& rq = tb.req[r];
-    const ShareSegment part = CUT ? share_segment(shares, npairs, pair, i, rq.Ls) : ShareSegment{unit, 0, rq.Ls, 0, 1};
+    ShareSegment part = {unit, 0, rq.Ls, 0, 1};
+    if constexpr (CUT) part = share_segment(shares, npairs, pair, i, rq.Ls);
     const int u = unit - tb.unit0_tc2[r];
     const int g = u / rq.tiles, kt = u % rq.tiles;
     const int key0 = kt * (int)kPairKeys + (int)rank * (int)kTile;
@@ -981,12 +986,9 @@ cudaError_t launch_score_tc(const void* Qw, const void* K, const Shape& sh, cons
                      scratch_bytes >= kSplitCountBytes + sizeof(float) * 2 * kPairKeys * (size_t)sh.L *
                                                              (size_t)std::min(tp.units2, pairs2);
   Shares shares;
-  if (!(split || per_layer) || tp.units2 > (int64_t)kShareUnits * pairs2 ||
-      !plan_shares(tp.req, tp.n_req, tp.units2, pairs2, &shares) ||
-      (tp.units2 <= pairs2 && !cuts_a_unit(shares, pairs2))) {
-    memset(&shares, 0, sizeof(shares));
-    shares.whole = 1;
-  }
+  const bool whole = !(split || per_layer) || tp.units2 > (int64_t)kShareUnits * pairs2 ||
+                     !plan_shares(tp.req, tp.n_req, tp.units2, pairs2, &shares) ||
+                     (tp.units2 <= pairs2 && !cuts_a_unit(shares, pairs2));
   cudaError_t e;
   if (!lse_nat) {
     const size_t smem1 = sizeof(P1Smem) + 1024;
@@ -1009,15 +1011,15 @@ cudaError_t launch_score_tc(const void* Qw, const void* K, const Shape& sh, cons
     if (e != cudaSuccess) return e;
   }
   const size_t smem2 = sizeof(P2Smem) + 1024;
-  auto colsum = [&](auto cut, int ctas) -> cudaError_t {
+  auto colsum = [&](auto cut, const auto& cuts, int ctas) -> cudaError_t {
     constexpr bool kCut = decltype(cut)::value;
     e = cudaFuncSetAttribute(score_colsum_tc_kernel<kCut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
     if (e != cudaSuccess) return e;
     ProfileScope ps("score_colsum_tc", st);
-    return launch_dep(score_colsum_tc_kernel<kCut>, dim3(ctas), dim3(kThreads), smem2, st, mq, mk, shares, sh, tb,
+    return launch_dep(score_colsum_tc_kernel<kCut>, dim3(ctas), dim3(kThreads), smem2, st, mq, mk, cuts, sh, tb,
                       static_cast<const float*>(nlse_pad), scores, scratch);
   };
-  return shares.whole ? colsum(std::false_type{}, 2 * tp.units2) : colsum(std::true_type{}, 2 * pairs2);
+  return whole ? colsum(std::false_type{}, NoShares{}, 2 * tp.units2) : colsum(std::true_type{}, shares, 2 * pairs2);
 }
 
 }  // namespace vc
