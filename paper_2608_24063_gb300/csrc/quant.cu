@@ -332,9 +332,13 @@ __global__ void __launch_bounds__(kQuantWarps * 32) quant_kernel(
   }
 }
 
-// 8 reconstructed channels (codes in the nibbles of q) to 8 adjacent outputs.
+// 8 reconstructed channels (codes in the nibbles of q) to 8 adjacent outputs of
+// a live row; in fp32 the whole warp calls it.  Two lanes hold 64 adjacent bytes of
+// an fp32 row: they swap halves, so that each store instruction writes whole
+// 32-byte sectors of it (8 requests of 6,000 tokens, d = 128: 186 us; with each
+// lane's own two 16-byte stores 267, with 4 channels a lane 199).
 template <typename T>
-__device__ __forceinline__ void store8(T* p, uint32_t q, const float (&scale)[8], const float (&lo)[8]) {
+__device__ __forceinline__ void store8(T* p, bool live, uint32_t q, const float (&scale)[8], const float (&lo)[8]) {
   float x[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {                // 2^23 + code, exact
@@ -350,8 +354,17 @@ __device__ __forceinline__ void store8(T* p, uint32_t q, const float (&scale)[8]
     }
     *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
   } else {
-    reinterpret_cast<float4*>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
-    reinterpret_cast<float4*>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
+    const bool odd = threadIdx.x & 1;
+    float y[4];                                // the other lane's half: its first if this one is even
+#pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = __shfl_xor_sync(0xffffffffu, odd ? x[j] : x[4 + j], 1);
+    // even: bytes 0-15 (its own) and 32-47 (the other's first half) of the 64;
+    // odd: 16-31 (the other's second half) and 48-63 (its own)
+    float4* at = reinterpret_cast<float4*>(p) - (odd ? 1 : 0);
+    if (live) {
+      at[0] = odd ? make_float4(y[0], y[1], y[2], y[3]) : make_float4(x[0], x[1], x[2], x[3]);
+      at[2] = odd ? make_float4(x[4], x[5], x[6], x[7]) : make_float4(y[0], y[1], y[2], y[3]);
+    }
   }
 }
 
@@ -372,6 +385,7 @@ __global__ void __launch_bounds__(kQuantWarps * 32) dequant_kernel(
     const uint8_t* __restrict__ Vc, const float2* __restrict__ Kp, const float2* __restrict__ Vp,
     T* __restrict__ Kh, T* __restrict__ Vh) {
   constexpr int LPR = D / 8, RPW = 32 / LPR;   // lanes of a row, rows of a step
+  constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;
   const int unit = blockIdx.x * kQuantWarps + (threadIdx.x >> 5);
   if (unit >= units) return;
   const int lane = threadIdx.x & 31, c0 = (lane % LPR) * 8, i0 = lane / LPR;
@@ -398,18 +412,21 @@ __global__ void __launch_bounds__(kQuantWarps * 32) dequant_kernel(
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    if (i0 + u * RPW < gr.nrows) store8(Kh + (gr.row + i0 + u * RPW) * D + c0, kq[u], ks, kl);
+    const int i = i0 + u * RPW;
+    if (kBf16 && i >= gr.nrows) continue;      // fp32: the whole warp stays, its lanes swap halves
+    store8(Kh + (gr.row + i) * D + c0, i < gr.nrows, kq[u], ks, kl);
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    if (i0 + u * RPW >= gr.nrows) continue;
+    const int i = i0 + u * RPW;
+    if (kBf16 && i >= gr.nrows) continue;
     float vs[8], vl[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       vs[j] = vp[u].x;
       vl[j] = vp[u].y;
     }
-    store8(Vh + (gr.row + i0 + u * RPW) * D + c0, vq[u], vs, vl);
+    store8(Vh + (gr.row + i) * D + c0, i < gr.nrows, vq[u], vs, vl);
   }
 }
 
