@@ -108,6 +108,21 @@ inline bool plan_shares(const TcReq* req, int n_req, int64_t units2, int pairs, 
   return true;
 }
 
+// Whether shares pay.  They fill the last wave of whole units, but pairs that start
+// inside different layers draw the window rows from the L2 at different times, and
+// split units leave sums in memory (not under layer-specific ranking).  So the last
+// wave has to leave a twelfth (a twentieth) of the pairs' time idle.  Whole calls, us,
+// whole units | shares, by units a pair and idle part: 1.3, 37% 250 | 226; 1.9, 5%
+// 319 | 326 (layer-specific 297 | 293); 2.6, 14% 462 | 452; 2.9, 4%, two ragged
+// requests 761 | 796; 3.3, 17% 622 | 602.  Past four units a pair equal requests
+// still gain (5.2, 14% 906 | 868; 8.3, 8% 2,026 | 1,987), ragged ones no more (5.4,
+// 11% 1,082 | 1,078; layer-specific 8.2, 9% 1,158 | 1,218), so the line lies there.
+constexpr int kShareUnits = 4;
+inline bool worth_sharing(int64_t units2, int pairs, bool per_layer) {
+  const int64_t slots = (units2 + pairs - 1) / pairs * pairs;
+  return units2 <= (int64_t)kShareUnits * pairs && (slots - units2) * (per_layer ? 20 : 12) > slots;
+}
+
 // Whether a cut lies inside a unit.  Without one, and with a pair for every unit,
 // whole units do the same with less to set up.
 inline bool cuts_a_unit(const Shares& s, int pairs) {

@@ -470,13 +470,13 @@ __global__ void lse_merge_kernel(Shape sh, Tables tb, int S, const float2* __res
 //
 // A launch with few units per resident pair is persistent: the (unit, layer)
 // sequence is cut into equal shares, one per pair, so a share may begin and end
-// inside a unit and no pair is idle in a last, partly filled wave.  Whole units
+// inside a unit and no pair is idle in a last, partly filled wave (worth_sharing).  Whole units
 // end in their scores.  The pairs that share a unit leave each layer's column
 // sums in the workspace, and the CTA that comes last (a count per unit and CTA
 // rank; nobody waits) adds them in layer order: the same additions in the same
 // order as for a whole unit, so the scores do not depend on the cuts.  A
 // longer sequence, or one without room for those sums, launches one pair per
-// unit (kShareUnits).
+// unit.
 //
 // Bound by the consumers, two warps per sub-partition: ~14 cycles a column
 // and warp pair where the exp2 unit needs 8 and the packed multiply-adds and
@@ -529,13 +529,6 @@ __device__ __forceinline__ float colsum_group(uint32_t col0, const float* nl_col
   return ((ps[0] + ps[1]) + (ps[2] + ps[3])) + ((ps[4] + ps[5]) + (ps[6] + ps[7]));
 }
 constexpr int kQStagesPair = 4;                 // Q ring of pass 2 (per CTA: 32 KB + 1 KB a stage)
-
-// Units per resident pair up to which a launch is cut into shares: the last
-// wave then wastes up to a quarter of the time.  Pairs that start inside
-// different layers draw the window rows from the L2 at different times, which
-// costs 10 to 20% a chunk: with 13 (72B shape) or 18 units a pair (ragged
-// batch of eight) shares took 4,357 against 4,288 us and 1,375 against 1,222.
-constexpr int kShareUnits = 4;
 
 struct Seg2 {                                   // layers [l0, l1) of one unit as this CTA sees it
   int64_t score;                                // first score of this CTA's keys (layer 0)
@@ -986,7 +979,7 @@ cudaError_t launch_score_tc(const void* Qw, const void* K, const Shape& sh, cons
                      scratch_bytes >= kSplitCountBytes + sizeof(float) * 2 * kPairKeys * (size_t)sh.L *
                                                              (size_t)std::min(tp.units2, pairs2);
   Shares shares;
-  const bool whole = !(split || per_layer) || tp.units2 > (int64_t)kShareUnits * pairs2 ||
+  const bool whole = !(split || per_layer) || !worth_sharing(tp.units2, pairs2, per_layer) ||
                      !plan_shares(tp.req, tp.n_req, tp.units2, pairs2, &shares) ||
                      (tp.units2 <= pairs2 && !cuts_a_unit(shares, pairs2));
   cudaError_t e;

@@ -44,6 +44,7 @@ extern "C" int plan(const int* req, int n_req, int pairs, int* cuts, int* out, i
     }
   return rows;
 }
+extern "C" int worth(int units2, int pairs, int per_layer) { return worth_sharing(units2, pairs, per_layer != 0); }
 """
 
 
@@ -54,7 +55,8 @@ def plan(tmp_path_factory):
     with open(src, "w") as f:
         f.write(HARNESS)
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, src, "-o", so], check=True)
-    fn = ctypes.CDLL(so).plan
+    lib = ctypes.CDLL(so)
+    fn = lib.plan
 
     def call(reqs, pairs):
         flat = (ctypes.c_int * (4 * len(reqs)))(*[x for q in reqs for x in q])
@@ -67,6 +69,7 @@ def plan(tmp_path_factory):
         return ([tuple(cuts[2 * p:2 * p + 2]) for p in range(pairs + 1)],
                 [tuple(out[6 * i:6 * i + 6]) for i in range(rows)])
 
+    call.worth = lib.worth
     return call
 
 
@@ -116,6 +119,13 @@ def test_random_batches(plan, seed):
                 for _ in range(rnd.choice([1, 1, 2, 5, 9]))]
         empties += _check(plan, reqs, rnd.choice([1, 2, 5, 74, 76, 128])) or 0
     assert empties > 0
+
+
+@pytest.mark.parametrize("units,layer,want", [(52, 0, True), (96, 0, True), (196, 0, True), (252, 0, True), (144, 0, False),
+                                              (144, 1, True), (218, 0, False), (218, 1, False), (76, 0, False),
+                                              (304, 0, False), (316, 0, False), (77, 0, True), (1, 0, True)])
+def test_shares_where_the_last_wave_idles(plan, units, layer, want):
+    assert bool(plan.worth(units, 76, layer)) == want
 
 
 def test_counts_are_cleared_before_pass_2_may_start_and_read_after_the_wait():
