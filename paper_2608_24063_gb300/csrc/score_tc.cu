@@ -51,7 +51,8 @@ using namespace tc;
 constexpr int kThreads = 384;                   // three warpgroups (warps 10 and 11 idle)
 // Registers per thread: the launch's 168 x 384 threads, moved from the third
 // warpgroup to the consumers, who hold 128 accumulators each (pass 2 at 168:
-// 154.5 us for n = 12,544 and 4,512 us for the 72B shape, now 149.7 and 4,288).
+// 154.4 us for n = 12,544 and 4,430 us for the 72B shape, now 150.5 and 4,315;
+// pass 1 the same either way; event times).
 constexpr int kConsumerRegs = 232, kOtherRegs = 40;
 static_assert(256 * kConsumerRegs + 128 * kOtherRegs <= 384 * 168, "the split fits what the launch gets");
 constexpr int kProducerWarp = 8, kMmaWarp = 9;
@@ -98,14 +99,13 @@ __device__ __forceinline__ float exp2_sum16(const float (&x)[16], float2 s, cons
 // of a unit.
 //
 // Bound by the consumers: per half tile and warp ~1,030 cycles of exps, 400 of
-// TMEM load and maximum, ~150 waiting for the slot (two warps share a
-// sub-partition's exp2 unit, which the 256 exps of both keep busy for 1,024).
+// TMEM load and maximum, ~150 waiting for the slot (clock stamps; two warps share
+// a sub-partition's exp2 unit, which the 256 exps of both keep busy for 1,024).
 // Slots of 128 columns, freed as soon as they are in registers, were slower
 // (153 us): an N = 128 MMA takes ~120 cycles, hardly less than an N = 256 one.
-// Measured, one unit per launched pair -> now: n = 3,136 58.4 -> 49.0 us, layer-
-// specific ranking at n = 12,544 144 -> 118 us, ragged batch 1,316 -> 1,285 us, 72B
-// shape 4,274 -> 4,110 us; n = 12,544 unchanged (147.5 us, three full waves either
-// way).
+// Measured (event times), one unit per launched pair -> now: n = 3,136 58.1 -> 47.3
+// us, n = 12,544 147.7 -> 140.4, layer-specific ranking 144.3 -> 118.3, ragged batch
+// 1,348 -> 1,257, 72B shape 4,456 -> 4,061.
 
 constexpr uint32_t kPairKeys = 256;             // keys per pass-1 tile (both CTAs)
 constexpr int kStagesPair = 4;                  // K ring of pass 1 (per CTA: 32 KB a stage)
@@ -480,9 +480,10 @@ __global__ void lse_merge_kernel(Shape sh, Tables tb, int S, const float2* __res
 //
 // Bound by the consumers, two warps per sub-partition: ~14 cycles a column
 // and warp pair where the exp2 unit needs 8 and the packed multiply-adds and
-// adds, at 4 cycles each, 8 as well.  Measured with one unit per launched pair
-// -> in shares: n = 3,136 (52 units on 76 pairs) 57.5 -> 51.8 us; n = 12,544 (196
-// units) 159.5 -> 149.7 us, layer-specific ranking 141.6 -> 123.4 us.
+// adds, at 4 cycles each, 8 as well.  Measured (event times), whole units in
+// every launch -> now: n = 3,136 (52 units on 76 pairs) 57.5 -> 52.7 us; n = 12,544
+// (196 units) 159.4 -> 150.5, layer-specific ranking 141.7 -> 125.0; whole units in
+// both: ragged batch 1,218 -> 1,235, 72B shape 4,422 -> 4,315.
 
 constexpr uint32_t kChunkRows = 256;            // window rows per pass-2 chunk (both CTAs)
 
