@@ -298,8 +298,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_partial_kernel(
 //
 // Measured on a GB300 (28 layers as a graph, 7B shape, n = 12,544 at 19% + 512
 // text rows; before: splits of 256 keys merged through global memory): one
-// request 382 -> 145 us a step, 16 requests 792 -> 495 us (5.4 TB/s of 6.8),
-// 4-bit cache of 16 requests 924 -> 528 us (556 with packed fp32 expansion).  A large
+// request 368 -> 145 us a step, 16 requests 790 -> 496 us (5.4 TB/s of 6.8),
+// 4-bit cache of 16 requests 923 -> 528 us (556 with packed fp32 expansion).  A large
 // layer runs at the memory rate (143 MB in 24 us) plus ~3 us that the launch, the
 // first loads and the merge take; the 4-bit form is bound by instruction latency
 // and issue (~1,400 warp instructions a tile, most of them the expansion, on two
