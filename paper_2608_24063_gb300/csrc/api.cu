@@ -243,7 +243,9 @@ struct Layout {
   // blocking, capturable in a CUDA graph); larger ones use one memcpy, and
   // then an upload of no bytes clears the status word, so that the kernels
   // after it always follow a kernel (their dependent launches order
-  // themselves on the kernel before them).
+  // themselves on the kernel before them).  Under capture a memcpy would leave
+  // the graph a pointer to this call's image, so a larger image then goes as
+  // several parameters.
   cudaError_t upload(uint8_t* ws, cudaStream_t st) const {
     const size_t bytes = table_end - table_begin;
     int32_t* status = reinterpret_cast<int32_t*>(ws + o_status);
@@ -255,7 +257,19 @@ struct Layout {
     }
     std::vector<uint8_t> img(bytes, 0);
     fill(img.data());
-    cudaError_t e = cudaMemcpyAsync(ws + table_begin, img.data(), bytes, cudaMemcpyHostToDevice, st);
+    cudaStreamCaptureStatus capture;
+    cudaError_t e = cudaStreamIsCapturing(st, &capture);
+    if (e != cudaSuccess) return e;
+    if (capture != cudaStreamCaptureStatusNone) {
+      TableImage im;
+      for (size_t at = 0; at < bytes && e == cudaSuccess; at += sizeof(im.bytes)) {
+        const size_t n = std::min(sizeof(im.bytes), bytes - at);
+        memcpy(im.bytes, img.data() + at, n);
+        e = launch_upload(im, (uint32_t)n, ws + table_begin + at, status, st);
+      }
+      return e;
+    }
+    e = cudaMemcpyAsync(ws + table_begin, img.data(), bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
     static const TableImage none = {};
     return launch_upload(none, 0u, ws + table_begin, status, st);
