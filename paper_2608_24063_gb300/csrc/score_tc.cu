@@ -1004,6 +1004,7 @@ cudaError_t launch_score_tc(const void* Qw, const void* K, const Shape& sh, cons
                    sh, tb, tp.S, static_cast<const float2*>(part), lse_nat, nlse_pad);
     if (e != cudaSuccess) return e;
   }
+  if (tp.units2 == 0) return cudaSuccess;      // no layer is scored (layer-specific ranking, all budgets 0)
   const size_t smem2 = sizeof(P2Smem) + 1024;
   auto colsum = [&](auto cut, const auto& cuts, int ctas) -> cudaError_t {
     constexpr bool kCut = decltype(cut)::value;
